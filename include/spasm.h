@@ -365,10 +365,11 @@ spasm_status spasm_inject_alloc_failure(int nth);
 /* Launch shape of the trajectory kernels (not in the paper: the tiling choices the autotuner
  * searches).  sphere_tiling: how a warp's lanes hold the (up to 64) sphere items of a
  * configuration, 0 strided (lane L holds items L and L + 32), 1 blocked (items 2L and 2L + 1);
- * particles_per_cta: particles one CTA optimises at once, 1 (8 warps) or 2 (16 warps, each
- * particle on its own 8 warps and shared-memory region; needs twice the shared memory).  The
+ * particles_per_cta: particles one CTA of 8 warps optimises at once, 1 (on all of them) or 2
+ * (each on its own 4 warps and shared-memory region; needs nearly twice the shared memory).  The
  * tiling reorders sums of the same terms (results agree to float32 rounding); the particles
- * per CTA change nothing in a particle's arithmetic. */
+ * per CTA change nothing in a particle's arithmetic.  A problem whose shape was never set leaves
+ * the particles per CTA to the library, launch by launch, from the particles and the sizes. */
 typedef struct {
     int sphere_tiling;
     int particles_per_cta;
@@ -419,7 +420,7 @@ typedef struct {
 } spasm_batch_config;
 /* per_fetch 1, ctas_per_sm 0, order 0, sphere_tiling 0, particles_per_cta 1. */
 spasm_status spasm_batch_default_config(spasm_batch_config* cfg);
-/* cfg NULL: the default schedule. */
+/* cfg NULL: the default schedule, with the particles per CTA left to the library. */
 spasm_status spasm_optimize_batch(spasm_problem_t* problems, int n, void* cuda_stream, const spasm_batch_config* cfg);
 /* Autotuner of the batched launch: places the problems not yet placed (stage 1, as above),
  * lifts them, times each trajectory shape (sphere tiling in {strided, blocked} x particles per

@@ -79,7 +79,7 @@ static void free_all(spasm_problem* pr) {
                     pr->d_idx, pr->d_sat, pr->d_nsat, pr->d_best, pr->d_place, pr->d_q, pr->d_lam,
                     pr->d_mu, pr->d_metrics, pr->d_tmasked, pr->d_tsat, pr->d_tnsat, pr->d_tbest, pr->d_rq,
                     pr->d_rcost, pr->d_rsucc, pr->d_cub64, pr->d_osph64, pr->d_rmet64, pr->d_tests, pr->d_sc, pr->d_chkacc,
-                    pr->d_ctl};
+                    pr->d_ctl, pr->d_rows, pr->d_work};
     for (void* p : ptrs)
         if (p) cudaFreeAsync(p, pr->stream);
     for (cudaEvent_t e : pr->ev)
@@ -137,6 +137,8 @@ static void for_each_buffer(spasm_problem* pr, int B, int C, int n_cub, int n_os
     f(pr->d_sc, 1);
     f(pr->d_chkacc, P);
     f(pr->d_ctl, 1);
+    f(pr->d_rows, (size_t)kTrajSlots * C * 16);
+    f(pr->d_work, 1);
 }
 
 extern "C" spasm_status spasm_problem_bytes(const spasm_obstacles* obs, const spasm_goal* goal, const spasm_params* prm,
@@ -387,6 +389,7 @@ static spasm_status create_problem_impl(const spasm_robot* robot, const spasm_ob
     if (e == cudaSuccess) e = cudaMemcpyAsync(pr->d_sc, &pr->sc, sizeof(Scalars), cudaMemcpyHostToDevice, pr->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(pr->d_err, 0, sizeof(int), pr->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(pr->d_chkacc, 0, sizeof(CheckAcc) * (size_t)prm->P, pr->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(pr->d_work, 0, sizeof(TrajWork), pr->stream);
     if (e == cudaSuccess) e = reset_loops(pr);
     if (e != cudaSuccess) {
         free_all(pr);
@@ -395,7 +398,7 @@ static spasm_status create_problem_impl(const spasm_robot* robot, const spasm_ob
     }
     pr->stats.h2d_bytes += (long long)(cub.size() * sizeof(float4) + osph.size() * sizeof(float4) +
                                        cub64.size() * sizeof(double) + osph64.size() * sizeof(double));
-    const size_t need = traj_smem_bytes(sc);
+    const size_t need = traj_cta_smem_bytes(sc, 1);
     int dev = 0, max_smem = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -619,6 +622,7 @@ extern "C" spasm_status spasm_traj_eval(spasm_problem_t pr, int n, const float* 
     io.lam = const_cast<float*>(lam);
     io.mu = const_cast<float*>(mu);
     io.L = L; io.grad = grad; io.groups = groups; io.h = h;
+    io.rows = pr->d_rows; io.work = pr->d_work;
     SPASM_CUDA(launch_traj(pr->sc, pr->tab, n, kTrajModeEval, io, pr->d_err, pr->stream));
     return SPASM_OK;
 }
@@ -630,6 +634,7 @@ extern "C" spasm_status spasm_traj_descend(spasm_problem_t pr, int n, float* q, 
     TrajIO io{};
     io.q = q; io.lam = lam; io.mu = mu; io.metrics = metrics; io.sat = sat;
     io.k_steps = k_steps; io.init_multipliers = init_multipliers;
+    io.rows = pr->d_rows; io.work = pr->d_work;
     SPASM_CUDA(launch_traj(pr->sc, pr->tab, n, kTrajModeDescend, io, pr->d_err, pr->stream));
     return SPASM_OK;
 }
@@ -668,8 +673,8 @@ extern "C" spasm_status spasm_set_kernel_config(spasm_problem_t pr, const spasm_
 extern "C" spasm_status spasm_traj_residency(spasm_problem_t pr, int* single, int* batched) {
     if (!pr || !single || !batched) return fail(SPASM_ERR_INVALID, "null argument");
     *single = traj_ctas_per_sm(pr->sc);
-    *batched = traj_batch_ctas_per_sm(traj_smem_bytes(pr->sc), pr->sc.sphere_tiling,
-                                      pr->sc.particles_per_cta == 2 ? 2 : 1);
+    const int ppc = traj_ppc(pr->sc, pr->sc.Q);
+    *batched = traj_batch_ctas_per_sm(traj_cta_smem_bytes(pr->sc, ppc), pr->sc.sphere_tiling, ppc);
     return SPASM_OK;
 }
 

@@ -123,13 +123,26 @@ void mark_placed(spasm_problem_t* prs, const std::vector<int>& todo) {
 // Work list of a batched trajectory launch over the problems `live` (in `order`).
 struct JobList {
     std::vector<TrajJob> jobs;
-    int n_items = 0;
-    size_t smem = 0;
+    int n_items = 0, ppc = 1;
+    size_t cta_bytes = 0;   // shared memory of a CTA with ppc particles of the largest problem
 };
 
+// ppc 0: the launcher's choice over all particles.
 JobList make_jobs(spasm_problem_t* prs, const std::vector<int>& live, int per_fetch, int mode, int k_steps,
-                  bool init_multipliers) {
+                  bool init_multipliers, int ppc) {
     JobList L;
+    if (ppc == 0) {
+        size_t two = 0;
+        long long particles = 0;
+        int blocks = 0;
+        for (int i : live) {
+            blocks = std::max(blocks, prs[i]->sc.B);
+            two = std::max(two, traj_cta_smem_bytes(prs[i]->sc, 2) + kBatchStaticSmem);
+            particles += prs[i]->sc.Q;
+        }
+        ppc = traj_auto_ppc(two, particles, blocks);
+    }
+    L.ppc = ppc;
     for (int i : live) {
         spasm_problem* pr = prs[i];
         TrajJob j{};
@@ -141,13 +154,14 @@ JobList make_jobs(spasm_problem_t* prs, const std::vector<int>& live, int per_fe
             j.io.tests = pr->d_tests;
             j.io.active = &pr->d_ctl->n_place;
         }
+        j.io.rows = pr->d_rows;
         j.io.k_steps = k_steps;
         j.io.init_multipliers = init_multipliers ? 1 : 0;
         j.err = pr->d_err;
         j.n = pr->sc.Q;
         j.first = L.n_items;
         L.n_items += (pr->sc.Q + per_fetch - 1) / per_fetch;
-        L.smem = std::max(L.smem, traj_smem_bytes(pr->sc));
+        L.cta_bytes = std::max(L.cta_bytes, traj_cta_smem_bytes(pr->sc, ppc));
         L.jobs.push_back(j);
     }
     return L;
@@ -183,14 +197,14 @@ spasm_status upload_jobs(const JobList& L, cudaStream_t s, DeviceJobs& d) {
     return SPASM_OK;
 }
 
-spasm_status batch_grid(const spasm_batch_config& cfg, size_t smem, int* grid) {
+spasm_status batch_grid(const spasm_batch_config& cfg, const JobList& L, int* grid) {
     int dev = 0, sms = 0;
     SPASM_CUDA(cudaGetDevice(&dev));
     SPASM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int resident = traj_batch_ctas_per_sm(smem, cfg.sphere_tiling, cfg.particles_per_cta);
+    const int resident = traj_batch_ctas_per_sm(L.cta_bytes, cfg.sphere_tiling, L.ppc);
     if (resident < 1) return fail(SPASM_ERR_INVALID, "batched trajectory kernel does not fit this shared-memory size");
     const int per_sm = cfg.ctas_per_sm > 0 ? std::min(cfg.ctas_per_sm, resident) : resident;
-    *grid = per_sm * sms;
+    *grid = std::min(per_sm * sms, kTrajSlots / L.ppc);
     return SPASM_OK;
 }
 
@@ -211,16 +225,15 @@ spasm::BatchLaunch::~BatchLaunch() {
 
 spasm_status spasm::prepare_batch(spasm_problem_t* prs, const std::vector<int>& order, const spasm_batch_config& cfg,
                                   cudaStream_t s, BatchLaunch& bl) {
-    SPASM_TRY(check_config(cfg));
-    JobList L = make_jobs(prs, order, cfg.per_fetch, kTrajModeDescend, 0, true);
+    JobList L = make_jobs(prs, order, cfg.per_fetch, kTrajModeDescend, 0, true, cfg.particles_per_cta);
     for (size_t k = 0; k < order.size(); ++k) L.jobs[k].io.k_steps = prs[order[k]]->sc.K_traj;
-    SPASM_TRY(batch_grid(cfg, L.smem, &bl.grid));
+    SPASM_TRY(batch_grid(cfg, L, &bl.grid));
     bl.host = std::move(L.jobs);
     bl.n_items = L.n_items;
-    bl.smem = L.smem;
+    bl.cta_bytes = L.cta_bytes;
     bl.per_fetch = cfg.per_fetch;
     bl.tiling = cfg.sphere_tiling;
-    bl.ppc = cfg.particles_per_cta;
+    bl.ppc = L.ppc;
     bl.s = s;
     SPASM_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&bl.jobs), sizeof(TrajJob) * bl.host.size(), s));
     SPASM_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&bl.next), sizeof(int), s));
@@ -231,7 +244,7 @@ spasm_status spasm::prepare_batch(spasm_problem_t* prs, const std::vector<int>& 
 spasm_status spasm::enqueue_batch(const BatchLaunch& bl, cudaStream_t s) {
     SPASM_CUDA(cudaMemsetAsync(bl.next, 0, sizeof(int), s));
     SPASM_CUDA(launch_traj_batch(bl.jobs, (int)bl.host.size(), bl.n_items, bl.per_fetch, kTrajModeDescend, bl.next,
-                                 bl.smem, bl.grid, s, bl.tiling, bl.ppc));
+                                 bl.cta_bytes, bl.grid, s, bl.tiling, bl.ppc));
     return SPASM_OK;
 }
 
@@ -251,8 +264,12 @@ extern "C" spasm_status spasm_optimize_batch(spasm_problem_t* prs, int n, void* 
     SPASM_TRY(check_batch(prs, n, cuda_stream));
     spasm_batch_config cfg;
     spasm_batch_default_config(&cfg);
-    if (cfg_in) cfg = *cfg_in;
-    SPASM_TRY(check_config(cfg));
+    if (cfg_in) {
+        cfg = *cfg_in;
+        SPASM_TRY(check_config(cfg));
+    } else {
+        cfg.particles_per_cta = 0;   // chosen by prepare_batch
+    }
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     std::vector<int> todo, all(n);
     for (int i = 0; i < n; ++i) {
@@ -335,22 +352,22 @@ extern "C" spasm_status spasm_batch_autotune(spasm_problem_t* prs, int n, void* 
     double shape_t = 1e300;
     for (int tiling = 0; tiling <= 1; ++tiling)
         for (int ppc = 1; ppc <= 2; ++ppc) {
-            JobList L = make_jobs(prs, job_order(prs, live, 0), 1, kTrajModeDescend, 0, true);
+            JobList L = make_jobs(prs, job_order(prs, live, 0), 1, kTrajModeDescend, 0, true, ppc);
             for (size_t k = 0; k < L.jobs.size(); ++k) {
                 L.jobs[k].io.k_steps = prs[job_order(prs, live, 0)[k]]->sc.K_traj;
                 L.jobs[k].io.tests = nullptr;   // the problems' counters are the solves'
             }
-            if (traj_batch_ctas_per_sm(L.smem, tiling, ppc) < 1) continue;   // two particles do not fit
+            if (traj_batch_ctas_per_sm(L.cta_bytes, tiling, ppc) < 1) continue;   // two particles do not fit
             spasm_batch_config c{1, 0, 0, tiling, ppc};
             int grid = 0;
-            SPASM_TRY(batch_grid(c, L.smem, &grid));
+            SPASM_TRY(batch_grid(c, L, &grid));
             DeviceJobs dj;
             SPASM_TRY(upload_jobs(L, s, dj));
             SPASM_TRY(lift_all());
             SPASM_CUDA(cudaMemsetAsync(dj.next, 0, sizeof(int), s));
             SPASM_CUDA(cudaEventRecord(e0, s));
-            SPASM_CUDA(launch_traj_batch(dj.jobs, (int)L.jobs.size(), L.n_items, 1, kTrajModeDescend, dj.next, L.smem,
-                                         grid, s, tiling, ppc));
+            SPASM_CUDA(launch_traj_batch(dj.jobs, (int)L.jobs.size(), L.n_items, 1, kTrajModeDescend, dj.next,
+                                         L.cta_bytes, grid, s, tiling, ppc));
             SPASM_CUDA(cudaEventRecord(e1, s));
             SPASM_CUDA(cudaEventSynchronize(e1));
             const double t = ev_ms(e0, e1);
@@ -366,9 +383,9 @@ extern "C" spasm_status spasm_batch_autotune(spasm_problem_t* prs, int n, void* 
         for (int pf : fetches)
             for (int per_sm : {0, 1}) {
                 spasm_batch_config c{pf, per_sm, order, tiling, ppc};
-                JobList L = make_jobs(prs, job_order(prs, live, order), pf, kTrajModeEval, 0, true);
+                JobList L = make_jobs(prs, job_order(prs, live, order), pf, kTrajModeEval, 0, true, ppc);
                 int grid = 0;
-                SPASM_TRY(batch_grid(c, L.smem, &grid));
+                SPASM_TRY(batch_grid(c, L, &grid));
                 DeviceJobs dj;
                 SPASM_TRY(upload_jobs(L, s, dj));
                 double t = 1e300;
@@ -376,7 +393,7 @@ extern "C" spasm_status spasm_batch_autotune(spasm_problem_t* prs, int n, void* 
                     SPASM_CUDA(cudaMemsetAsync(dj.next, 0, sizeof(int), s));
                     SPASM_CUDA(cudaEventRecord(e0, s));
                     SPASM_CUDA(launch_traj_batch(dj.jobs, (int)L.jobs.size(), L.n_items, pf, kTrajModeEval, dj.next,
-                                                 L.smem, grid, s, tiling, ppc));
+                                                 L.cta_bytes, grid, s, tiling, ppc));
                     SPASM_CUDA(cudaEventRecord(e1, s));
                     SPASM_CUDA(cudaEventSynchronize(e1));
                     if (rep > 0) t = ev_ms(e0, e1);

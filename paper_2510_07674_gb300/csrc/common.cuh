@@ -27,7 +27,9 @@ constexpr float kPi = 3.14159265358979323846f;
 
 // Scalars, robot tables and block tables: passed by value as a __grid_constant__ kernel
 // parameter (about 3 KB, well inside the 32 KB parameter space of CUDA 12.1+).
-struct Scalars {
+// TrajScalars is the part the stage-2 evaluation reads again and again; the batched
+// trajectory kernel keeps a copy of it (1.4 KB) in shared memory per particle group.
+struct TrajScalars {
     int B, S, C, NR;                 // blocks, steps per segment (W-1), configurations, residuals
     int n_rsph, n_cub, n_osph;       // robot spheres, env cuboids, env spheres
     int K_lin, K_quad, K_traj, K_al, K_ik;
@@ -37,8 +39,6 @@ struct Scalars {
     float qlo[7], qhi[7];
     float ee_R[9], ee_p[3];
     float q_home[7];
-    float4 rsph[kMaxRobotSpheres];   // x, y, z, r in the link frame
-    int rlink[kMaxRobotSpheres];     // 0 = base
     float4 lbox_c[8], lbox_h[8];     // per link: box of its spheres in the link frame (centre, half
                                      // extents, slightly padded); half.x < 0 when the link has none
     float sweep[7];                  // per joint: bound on the distance from its axis to any robot or
@@ -59,12 +59,18 @@ struct Scalars {
     int ik_mode;                     // lift IK: 0 damped least squares, 1 analytic (Franka joint layout)
     int sphere_tiling;               // trajectory kernels: sphere items per lane, 0 strided (lane + 32 k),
                                      // 1 blocked (2 lane + k); the same terms, summed in another order
-    int particles_per_cta;           // trajectory kernels: particles a CTA runs at once, 1 or 2 (0 = 1)
+    int particles_per_cta;           // trajectory kernels: particles a CTA runs at once, 1 or 2, or 0 for
+                                     // the launcher's choice (traj_auto_ppc)
+    int kind;                        // GoalKind
     unsigned long long seed;
+};
+
+struct Scalars : TrajScalars {
+    float4 rsph[kMaxRobotSpheres];   // x, y, z, r in the link frame
+    int rlink[kMaxRobotSpheres];     // 0 = base
     // packing goal (the appendix's Tetris problem), kind = kKindPack: block i is a polyomino
     // of unit cubes of edge cell_size centred at cell[cell_start[i] .. cell_start[i+1]) in
     // its frame; the walls are the environment cuboids; z_star is the resting height
-    int kind;
     int n_cells;
     int cell_start[kMaxB + 1];
     signed char cell_block[kMaxCells];   // block of each cell
@@ -155,6 +161,18 @@ __device__ __forceinline__ float warp_min(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
+}
+
+// Smallest / largest of the lanes' values (NaN ignored, as fminf / fmaxf) in one instruction.
+__device__ __forceinline__ float warp_fmin(float v) {
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float warp_fmax(float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
 }
 
 // ------------------------------------------------------------------------------ geometry
@@ -270,7 +288,7 @@ __device__ __forceinline__ void sincos_t(double x, double* s, double* c) { sinco
 
 // Tool frame from frame 7: R_tool = R7 ee_R, p_tool = o7 + R7 ee_p.
 template <typename T>
-__device__ __forceinline__ void tool_frame(const Scalars& sc, const T R7[9], const T o7[3], T Rt[9], T pt[3]) {
+__device__ __forceinline__ void tool_frame(const TrajScalars& sc, const T R7[9], const T o7[3], T Rt[9], T pt[3]) {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
 #pragma unroll
@@ -301,7 +319,7 @@ __device__ __forceinline__ void fk_full(const Scalars& sc, const T q[7], T R[8][
 // Block frame held by the tool (top-down grasp): R_blk = R_tool diag(1,-1,-1),
 // p_blk = p_tool + (hz + grasp_off) z_tool.
 template <typename T>
-__device__ __forceinline__ void held_block(const Scalars& sc, int b, const T Rt[9], const T pt[3], T Rb[9], T pb[3]) {
+__device__ __forceinline__ void held_block(const TrajScalars& sc, int b, const T Rt[9], const T pt[3], T Rb[9], T pb[3]) {
     T off = (T)sc.half[b].z + (T)sc.grasp_off;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {

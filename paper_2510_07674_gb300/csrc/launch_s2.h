@@ -4,6 +4,12 @@
 
 namespace spasm {
 
+// Work counters of a persistent trajectory launch, zero between launches: the particles handed
+// out after each group's first, and the groups that are done.
+struct TrajWork {
+    int next, done;
+};
+
 // Buffers of one trajectory-kernel launch (device pointers; any may be null unless noted).
 struct TrajIO {
     float* q;          // [n][C][8] joint configurations (required); updated by a descent
@@ -22,7 +28,13 @@ struct TrajIO {
     int init_multipliers;   // descent starts from lambda = 0, mu = mu0
     const int* active;  // optional device word: when it holds 0 or less the launch does nothing (the
                         // trajectory stage of a problem whose stage 1 found no placement)
+    float* rows;        // [kTrajSlots][C][16] scratch (required): the collision gradient rows of the
+                        // particle each resident group works on
+    TrajWork* work;   // the launch's work counters (required by launch_traj), zero between launches
 };
+// Particle groups resident at once: two CTAs of two groups on each of 152 SMs; a launch on a
+// part with more SMs keeps to this many.
+constexpr int kTrajSlots = 608;
 enum TrajModeHost { kTrajModeEval = 0, kTrajModeDescend = 1, kTrajModeCheck = 2 };
 
 // One problem of a batched trajectory launch (device array, sorted by `first`).
@@ -35,7 +47,10 @@ struct TrajJob {
     int first;           // index of the problem's first work item
 };
 
-size_t traj_smem_bytes(const Scalars& sc);
+// Particles per CTA of a launch of that many particles: the problem's setting, or the
+// launcher's choice (traj_auto_ppc, given the shared memory of a CTA with two particles and the blocks).
+int traj_ppc(const TrajScalars& sc, long long particles);
+int traj_auto_ppc(size_t cta_bytes_2, long long particles, int blocks);
 // IK at grasp/place poses + interpolation; particle p lifts placement p % n_place.  With
 // ctl != nullptr the attempt counter, the placement count and the Philox key are read on the
 // device (ctl->t_attempt, ctl->n_place, ctl->seed) in place of `attempt`, `n_place` and
@@ -44,18 +59,20 @@ cudaError_t launch_lift(const Scalars& sc, int n, const float* place, int n_plac
                         cudaStream_t st, const LoopCtl* ctl = nullptr);
 cudaError_t launch_traj(const Scalars& sc, DevTables t, int n, int mode, const TrajIO& io, int* err, cudaStream_t st);
 // Persistent batched launch over jobs[0..n_jobs) (n_items work items of per_fetch particles;
-// *next must be 0); smem_bytes = the largest traj_smem_bytes of the jobs.
-// tiling, ppc: the sphere tiling (Scalars::sphere_tiling) and the particles per CTA
-// (Scalars::particles_per_cta) of the launch, the same for every job.
+// *next must be 0); cta_bytes = the largest traj_cta_smem_bytes of the jobs; grid x ppc <=
+// kTrajSlots.  tiling, ppc: the sphere tiling (Scalars::sphere_tiling) and the particles per CTA
+// (1 or 2) of the launch, the same for every job.
 cudaError_t launch_traj_batch(const TrajJob* jobs, int n_jobs, int n_items, int per_fetch, int mode, int* next,
-                              size_t smem_bytes, int grid, cudaStream_t st, int tiling = 0, int ppc = 1);
-// Resident CTAs per SM of the batched kernel at that per-particle shared-memory size (0 on error
+                              size_t cta_bytes, int grid, cudaStream_t st, int tiling, int ppc);
+// Upper bound on the batched kernel's static shared memory (its copies of two problems' constants).
+constexpr size_t kBatchStaticSmem = 2 * (sizeof(TrajScalars) + sizeof(TrajIO) + 8) + 64;
+// Resident CTAs per SM of the batched kernel at that shared-memory size of a CTA (0 on error
 // or when it does not fit).
-int traj_batch_ctas_per_sm(size_t smem_bytes, int tiling = 0, int ppc = 1);
+int traj_batch_ctas_per_sm(size_t cta_bytes, int tiling, int ppc);
 // Resident CTAs per SM of the per-problem trajectory kernel for this problem's sizes and launch
 // shape (0 if it does not fit).
-int traj_ctas_per_sm(const Scalars& sc);
+int traj_ctas_per_sm(const TrajScalars& sc);
 // Dynamic shared memory of one trajectory CTA with ppc particles.
-size_t traj_cta_smem_bytes(const Scalars& sc, int ppc);
+size_t traj_cta_smem_bytes(const TrajScalars& sc, int ppc);
 
 }  // namespace spasm

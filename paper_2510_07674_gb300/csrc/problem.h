@@ -49,6 +49,8 @@ struct spasm_problem {
     int *d_tsat = nullptr, *d_tnsat = nullptr, *d_tbest = nullptr;
     float *d_rq = nullptr, *d_rcost = nullptr;   // returned solutions
     int* d_rsucc = nullptr;
+    float* d_rows = nullptr;             // the trajectory kernel's gradient rows (kTrajSlots x C x 16)
+    spasm::TrajWork* d_work = nullptr;   // and work counters
     unsigned long long* d_tests = nullptr;   // [tests run, configurations culled] by the trajectory kernel
     bool optimized = false;
     int n_found = 0, traj_attempts = 0;
@@ -136,14 +138,15 @@ struct BatchLaunch {
     int* next = nullptr;
     cudaStream_t s = nullptr;
     int n_items = 0, grid = 0, per_fetch = 1, tiling = 0, ppc = 1;
-    size_t smem = 0;
+    size_t cta_bytes = 0;
     BatchLaunch() = default;
     BatchLaunch(const BatchLaunch&) = delete;
     BatchLaunch& operator=(const BatchLaunch&) = delete;
     ~BatchLaunch();
 };
 // Builds and uploads (on s, asynchronously) the work list of problems prs[order[k]], each with
-// its own K_traj steps and its placement count as the gate.
+// its own K_traj steps and its placement count as the gate.  cfg.particles_per_cta 0 leaves
+// that choice to the launcher (traj_auto_ppc over all particles).
 spasm_status prepare_batch(spasm_problem_t* prs, const std::vector<int>& order, const spasm_batch_config& cfg,
                            cudaStream_t s, BatchLaunch& bl);
 // Enqueues the launch (resetting its work counter first).

@@ -121,6 +121,7 @@ void scheduler_loop(spasm_server* sv) {
     std::vector<std::shared_ptr<Request>> active;
     spasm_batch_config cfg;
     spasm_batch_default_config(&cfg);
+    cfg.particles_per_cta = 0;   // chosen per epoch
     for (;;) {
         std::vector<std::shared_ptr<Request>> admitted;
         {

@@ -16,12 +16,13 @@ struct PlaceOut {
     float maxpen, maxD, maxdz;           // satisfying metrics
 };
 
-// Per-warp shared scratch of the placement evaluation.
-struct PlaceScratch {
-    float4 bc[kMaxB][4];     // block cuboids
+// Per-warp shared scratch of the placement evaluation: the support factors, and in stage 1
+// the block cuboids (stage 2 keeps its own).
+struct StackScratch {
     float stab[kMaxB][4];    // a_i dD_i/dv (x, y), a_i dD_i/dyaw, D_i
-    float e[kMaxB];          // height residuals
-    float D[kMaxB];
+};
+struct PlaceScratch : StackScratch {
+    float4 bc[kMaxB][4];     // block cuboids
 };
 
 // Coefficient modes of the gradient: stage-1 cost (a = w_stable, b = 2 w_height e,
@@ -33,12 +34,12 @@ enum PlaceMode { kPlaceForward = 0, kPlaceStage1 = 1, kPlaceExplicit = 2, kPlace
 // Per-block terms of the tower (lane i < B owns block i): height residual e_i, support
 // distance D_i and the block cuboids in ps.  With mode kPlaceStage1 or kPlaceExplicit, sets
 //   g = sum_i a_i dD_i/dx + sum_i b_i de_i/dx   (the collision part is added by the caller);
-// with kPlaceUnit, leaves dD_i/d(centre of mass, yaw) in ps.stab for place_stack_grad and
-// writes no block cuboids.
+// with kPlaceUnit, leaves dD_i/d(centre of mass, yaw) in ps.stab for place_stack_grad.
 // x, g: per-warp shared arrays of 4B floats.  Must be called by all 32 lanes of the warp.
-__device__ __forceinline__ void place_stack_warp(const Scalars& sc, const float* x, int mode, const float* a_in,
-                                                 const float* b_in, float* g, PlaceScratch& ps, float& my_D,
-                                                 float& my_e) {
+// bc: the block cuboids, written here or, in mode kPlaceUnit, already those of x.
+__device__ __forceinline__ void place_stack_warp(const TrajScalars& sc, const float* x, int mode, const float* a_in,
+                                                 const float* b_in, float* g, StackScratch& ps, float4 (*bc)[4],
+                                                 float& my_D, float& my_e) {
     const int lane = threadIdx.x & 31;
     const int B = sc.B;
     const bool want_grad = mode != kPlaceForward;
@@ -46,16 +47,15 @@ __device__ __forceinline__ void place_stack_warp(const Scalars& sc, const float*
     if (lane < B) {
         const int i = lane;
         my_e = x[4 * i + 2] - sc.zt[i];
-        ps.e[i] = my_e;
-        if (mode != kPlaceUnit)   // the stage-2 caller keeps its own placed cuboids
-            block_cuboid(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3], sc.half[i], ps.bc[i]);
+        if (mode != kPlaceUnit)
+            block_cuboid(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3], sc.half[i], bc[i]);
         float sx = 0.f, sy = 0.f, dvx = 0.f, dvy = 0.f, dyaw = 0.f;
         if (i + 1 < B) {
             const int n_above = B - 1 - i;
+#pragma unroll 1
             for (int j = i + 1; j < B; ++j) { sx += x[4 * j]; sy += x[4 * j + 1]; }
             const float mx = sx / (float)n_above, my = sy / (float)n_above;
-            float s, c;
-            sincosf(x[4 * i + 3], &s, &c);
+            const float c = bc[i][1].x, s = bc[i][1].y;   // of the yaw
             const float vx = mx - x[4 * i], vy = my - x[4 * i + 1];
             const float ux = c * vx + s * vy, uy = -s * vx + c * vy;       // Rz(-yaw) v
             const float ex = fmaxf(fabsf(ux) - sc.half[i].x, 0.f), ey = fmaxf(fabsf(uy) - sc.half[i].y, 0.f);
@@ -69,12 +69,12 @@ __device__ __forceinline__ void place_stack_warp(const Scalars& sc, const float*
             }
         }
         ps.stab[i][0] = dvx; ps.stab[i][1] = dvy; ps.stab[i][2] = dyaw; ps.stab[i][3] = my_D;
-        ps.D[i] = my_D;
     }
     __syncwarp();
     if (want_grad && mode != kPlaceUnit && lane < B) {
         const int i = lane;
         float gx = -ps.stab[i][0], gy = -ps.stab[i][1];
+#pragma unroll 1
         for (int k = 0; k < i; ++k) {
             const float inv = 1.f / (float)(B - 1 - k);
             gx += ps.stab[k][0] * inv;
@@ -88,13 +88,14 @@ __device__ __forceinline__ void place_stack_warp(const Scalars& sc, const float*
 
 // The gradient place_stack_warp writes in mode kPlaceExplicit, from the factors its kPlaceUnit
 // pass left in ps (a_i dD_i/d... = a_i times the unit factor, in the same order of operations).
-__device__ __forceinline__ void place_stack_grad(const Scalars& sc, const PlaceScratch& ps, const float* a_in,
+__device__ __forceinline__ void place_stack_grad(const TrajScalars& sc, const StackScratch& ps, const float* a_in,
                                                  const float* b_in, float* g) {
     const int lane = threadIdx.x & 31;
     const int B = sc.B;
     if (lane < B) {
         const int i = lane;
         float gx = -(a_in[i] * ps.stab[i][0]), gy = -(a_in[i] * ps.stab[i][1]);
+#pragma unroll 1
         for (int k = 0; k < i; ++k) {
             const float inv = 1.f / (float)(B - 1 - k);
             gx += (a_in[k] * ps.stab[k][0]) * inv;
@@ -118,7 +119,7 @@ __device__ __forceinline__ void place_eval_warp(const Scalars& sc, const float4*
     const int B = sc.B;
     const bool want_grad = mode != kPlaceForward;
     float my_D, my_e;
-    place_stack_warp(sc, x, mode, a_in, b_in, g, ps, my_D, my_e);
+    place_stack_warp(sc, x, mode, a_in, b_in, g, ps, ps.bc, my_D, my_e);
 
     // -- collisions: items (block j, sphere m)
     const float s_coll = mode == kPlaceStage1 ? sc.w_coll : s_coll_in;

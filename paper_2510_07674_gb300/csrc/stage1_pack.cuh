@@ -33,7 +33,6 @@ __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const fl
     if (lane < B) {
         const int i = lane;
         my_e = x[4 * i + 2] - sc.z_star;
-        ps.e[i] = my_e;
         block_cuboid(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3], half, ps.bc[i]);
         if (want_grad) {
             const float b = mode == kPlaceStage1 ? sc.w_height * (my_e > 0.f ? 1.f : (my_e < 0.f ? -1.f : 0.f)) : b_in[i];

@@ -17,7 +17,7 @@ __host__ __device__ __forceinline__ int t_place(int S, int b) { return (2 * b + 
 //   [5B+2b..+1] place of block b: roll, pitch                        (w_start)
 //   [7B+b] height residual, [8B+b] CoM distance,                    (w_height, w_stable)
 //   [9B] placement collisions, [9B+1] C_arm, [9B+2] C_block.         (w_coll, w_arm, w_block)
-__device__ __forceinline__ float residual_sqrt_weight(const Scalars& sc, int r) {
+__device__ __forceinline__ float residual_sqrt_weight(const TrajScalars& sc, int r) {
     const int B = sc.B;
     const int k = r < 7 * B ? 0 : r < 8 * B ? 1 : r < 9 * B ? 2 : r == 9 * B ? 3 : r == 9 * B + 1 ? 4 : 5;
     return sc.sqw[k];
