@@ -42,19 +42,24 @@ __device__ __forceinline__ void grp_sync() {
     else asm volatile("bar.sync 2, %0;" ::"n"(kGrpThreads<kPpc>) : "memory");
 }
 
-// Cached cull.  When a chunk's cull finds no candidate for any of its configurations, it
-// also returns the chunk's clearances: the smallest separation (largest per-axis gap) between
-// any of its link boxes and any static box that could touch it (the environment, blocks at
-// their initial poses), and the same for the placed blocks, which move: the top one (the
+// Cached cull.  When no sphere of a chunk penetrates a static obstacle (the environment, blocks
+// at their initial poses), its cull and tests also return the chunk's static clearance: the
+// smallest separation (largest per-axis gap) between any of its link boxes and any static box
+// that could touch it, and for the obstacles its spheres were tested against the smallest
+// sphere-level gap of those tests.  The same for the placed blocks, which move: the top one (the
 // highest block placed before the chunk's last block) on its own, the ones below it together.
-// Later iterations skip the chunk (kinematics, cull and tests: its terms are zero) while the
-// bound on how far its spheres moved since stays below the static clearance, plus the top
-// block's own motion since below the clearance to it, and plus a bound on how far any one of
-// the blocks below the top one moved below the clearance to those, so the skipped work is
-// exactly the work whose result is zero.  A chunk whose configurations have
-// candidates but whose spheres all miss them (no penetration anywhere: its terms are zero as
-// well) is kept the same way; for the obstacles its spheres were tested against, its
-// clearance is the smallest sphere-level gap those tests found.
+// Later iterations skip the static half while the bound on how far the chunk's spheres moved
+// since stays below the static clearance, and the moving half while that bound plus the top
+// block's own motion since stays below the clearance to it, and plus a bound on how far any one
+// of the blocks below the top one moved below the clearance to those: the skipped work is exactly
+// work whose result is zero.  A chunk with both halves skipped needs no kinematics; one with one
+// half evaluated again keeps the other's clearance less the motion so far.  (Most chunks that
+// have to be looked at again have come due for the placed blocks' motion alone, which leaves one
+// word of boxes to cull.)
+// A chunk's state byte: how many of its configurations had a candidate when it was last evaluated,
+// the halves that this evaluation may skip, the halves without a penetration.
+constexpr int kStateCand = 7, kStateSkipStatic = 16, kStateSkipMoving = 32, kStateZeroStatic = 64, kStateZeroMoving = 128;
+constexpr int kStateZero = kStateZeroStatic | kStateZeroMoving;
 constexpr float kClearSlack = 1e-5f;   // FP32 rounding of the boxes, metres
 
 // Work queue of an evaluation: its items (the chunks, the residual jobs, the slices of the
@@ -68,7 +73,7 @@ __device__ __forceinline__ void fx_add(long long* acc, float v) {
 }
 __device__ __forceinline__ float fx_value(long long a) { return __ll2float_rn(a) * (1.f / kFix); }
 constexpr int kPlaceUnits = (8 * kMaxB + 31) / 32;   // slices of 32 block spheres of the placed tower
-constexpr int kResidualJobs = 2;                      // placement residuals; start residuals
+constexpr int kResidualJobs = 1;                      // the placement residuals
 
 // The obstacles of the cull, in words of 32 boxes (padded with empty ones): the environment's
 // cuboids, its spheres, then one word of blocks, bit k the placed block k and bit 16 + k block k
@@ -100,9 +105,8 @@ struct TShared {
     float pose[4 * kMaxB];   // placed poses (x, y, z, yaw)
     float g4[4 * kMaxB];     // dL/d(placed pose)
     float h[kMaxNR], lam[kMaxNR], s[kMaxNR];
-    // gradient rows of the grasp (b) and place (B + b) configurations; until the gradient pass
-    // overwrites them, their first 6 floats hold the residual pass's (w_roll, w_pitch) of that block frame
-    alignas(16) float extra[2 * kMaxB][8];
+    float rpt[2 * kMaxB][6];           // (w_roll, w_pitch) of the block frame at special configuration e
+                                       // (2 b: grasp of block b, 2 b + 1: place)
     float pg[kMaxB][4];                // dC_coll/d(placed pose j), sphere side (from the slice holding block j)
     float pgc[kPlaceUnits][kMaxB][4];  // dC_coll/d(placed pose i), cuboid side of block pairs, per slice
     float pcu[kPlaceUnits][2];         // per slice: sum and maximum of the tower's penetrations
@@ -113,11 +117,15 @@ struct TShared {
     float4 dh[8];            // joint j: cos alpha, sin alpha, a, d (per-lane reads in the kinematics)
     float th0[8];            // joint offsets
     float4 lbc[8], lbh[8];   // link-frame boxes of each link's spheres (centre, half extents)
-    float s_arm, s_blk, mu, L, inv_S;
+    float mu, L, inv_S;
+    float inv_above[kMaxB];       // 1 / (blocks above block k)
     float pose_prev[4 * kMaxB];   // placed poses of the previous evaluation
     // chunks to evaluate by tier (kChunk .. 1 configurations with candidates at the last cull, then the
     // candidate-free ones to cull again)
-    unsigned char active[kChunk + 1][(kMaxC + kChunk - 1) / kChunk];
+    union {
+        unsigned char active[kChunk + 1][(kMaxC + kChunk - 1) / kChunk];
+        float4 partial[2 * kMaxB][2];   // traj_step: the special configurations' gradients without their own rows
+    };
     int n_tier[kChunk + 1];       // their counts
     unsigned hit[kMaxC / 32];     // bit t - 1: configuration t has gradient rows this evaluation
     float blk_cum[kMaxB];         // [k]: sum over the evaluations of the largest motion among the placed blocks 0..k
@@ -149,8 +157,7 @@ __host__ __device__ inline int t_n_chunks(int C) { return (C - 1 + kChunk - 1) /
 // cached cull state: per configuration the motion bound since its chunk's last cull; per
 // chunk, at that cull, the motion bound of the placed blocks below its top block and the top
 // block's own motion, its (static, moving) clearances as an fp16 pair, its fp16 clearance to
-// the top block and how many of its configurations had a candidate (0: none, the chunk's cull
-// is cacheable)
+// the top block and its state (kState*)
 __host__ __device__ inline size_t t_cache_offset(int n_cub, int n_osph, int C, int B, int warps) {
     return (t_sp_offset(n_cub, n_osph, C, warps) + (size_t)2 * B * sizeof(SpecialFrames) + 15) & ~(size_t)15;
 }
@@ -353,19 +360,20 @@ __device__ __forceinline__ float warp_sums(float v[N]) {
 // gradients of configuration t to rows[16 t ..] (arm group, then block group, 8 floats each)
 // where it penetrates something, marks those in sh.hit and accumulates placed-pose derivatives.
 // seg_l: the segment of configuration t0 + lane / 8.
-// Returns whether the chunk's collision terms are zero (no candidate, or candidates that no
-// sphere penetrates); then `clearance` / `clearance_top` / `clearance_moving` bound from below
-// how far any of its spheres is from a static box / the top placed block it could touch (the
-// block below the chunk's last block) / the other placed blocks: the gaps between link boxes
-// and the boxes apart from them, and the sphere-level gaps of the tests that ran.
+// skip (kStateSkip*): the half (static obstacles, placed blocks) known to be clear of the chunk.
+// Returns the halves without a penetration (kStateZero*); for those evaluated, `clearance` /
+// `clearance_top` / `clearance_moving` bound from below how far any of the chunk's spheres is
+// from a static box / the top placed block it could touch (the block below the chunk's last
+// block) / the other placed blocks: the gaps between link boxes and the boxes apart from them,
+// and the sphere-level gaps of the tests that ran.
 // The environment and the blocks share one cull loop and one test loop, and the kernel keeps
 // its other loops rolled: with four particles per SM in different phases the instruction cache
 // is what the warps compete for.
 template <int kTile>
-__device__ __forceinline__ bool chunk_collisions(const TrajScalars& sc, const LaneSpheres& ls,
+__device__ __forceinline__ int chunk_collisions(const TrajScalars& sc, const LaneSpheres& ls,
                                                  const float4* __restrict__ cub, const float4* __restrict__ osph,
                                                  const float4* aabb, TShared& sh, TWarp& tw, float* rows, int t0,
-                                                 int nc, int seg_l, bool grad, const float* lane_box, float& acc_arm,
+                                                 int nc, int seg_l, int skip, bool grad, const float* lane_box, float& acc_arm,
                                                  float& acc_blk, float& acc_max, int& n_cand, float& clearance,
                                                  float& clearance_moving, float& clearance_top) {
     const int lane = threadIdx.x & 31;
@@ -394,15 +402,17 @@ __device__ __forceinline__ bool chunk_collisions(const TrajScalars& sc, const La
     auto context = [](int below, int above) {   // placed blocks k < below, initial poses k > above
         return ((1u << below) - 1u) | (0xfffe0000u << above);
     };
-    const unsigned ctx_l = context(b_lane, b_lane), ctx_chunk = context(b_last, b_first);
+    const unsigned halves = (skip & kStateSkipStatic ? 0u : 0xffff0000u) | (skip & kStateSkipMoving ? 0u : 0x0000ffffu);
+    const unsigned ctx_l = context(b_lane, b_lane) & halves, ctx_chunk = context(b_last, b_first) & halves;
     // the highest placed block a configuration of the chunk can touch: it moves by its own motion,
     // the blocks below it by at most the largest motion among them
     const int top = b_last - 1;
     const int n_cw = t_cub_words(sc.n_cub), n_w = t_words(sc.n_cub, sc.n_osph);
+    const int wd0 = skip & kStateSkipStatic ? n_w - 1 : 0;
     float clear = 3.4e38f, clear_m = 3.4e38f;
     uint32_t any = 0u;
 #pragma unroll 1
-    for (int wd = 0; wd < n_w; ++wd) {
+    for (int wd = wd0; wd < n_w; ++wd) {
         const bool blocks = wd == n_w - 1;
         const float4* box = aabb + 64 * wd;
         const float4 clo = box[2 * lane], chi = box[2 * lane + 1];
@@ -466,6 +476,7 @@ __device__ __forceinline__ bool chunk_collisions(const TrajScalars& sc, const La
     // move relative to static boxes and are left out of gap_s.
     n_cand = 0;
     unsigned hits = 0u;   // bit c: configuration c penetrates something
+    bool hit_s = false, hit_m = false;
     int visits = 0;
     float gap_s = 3.4e38f, gap_m = 3.4e38f, gap_t = 3.4e38f;
     unsigned tests = 0u;
@@ -489,7 +500,7 @@ __device__ __forceinline__ bool chunk_collisions(const TrajScalars& sc, const La
         visits = 0;
 
 #pragma unroll 1
-        for (int wd = 0; wd < n_w; ++wd) {
+        for (int wd = wd0; wd < n_w; ++wd) {
             const bool blocks = wd == n_w - 1;
             unsigned m = tw.mask[ci][wd];
             visits += __popc(m);
@@ -510,7 +521,7 @@ __device__ __forceinline__ bool chunk_collisions(const TrajScalars& sc, const La
                         float ax, ay, az;
                         const float pen = pen_sphere<float>(cx[sl], cy[sl], cz[sl], rr[sl], os, ax, ay, az);
                         if (pen > 0.f) {
-                            any_hit = true;
+                            any_hit = hit_s = true;
                             pen_sum[sl] += pen;
                             acc_max = fmaxf(acc_max, pen);
                             gx[sl] += ax; gy[sl] += ay; gz[sl] += az;
@@ -554,6 +565,8 @@ __device__ __forceinline__ bool chunk_collisions(const TrajScalars& sc, const La
                     }
                 }
                 any_hit |= hit;
+                if (placed) hit_m |= hit;
+                else hit_s |= hit;
                 if (grad && placed && __any_sync(0xffffffffu, hit)) {
                     const float d = warp_sums<8>(d8);   // lane 4 i: value i
                     if ((lane & 3) == 0) fx_add(&sh.fx_wr[lane >> 4][bit][(lane >> 2) & 3], d);
@@ -603,24 +616,34 @@ __device__ __forceinline__ bool chunk_collisions(const TrajScalars& sc, const La
         tw.count[1] += (unsigned)nc;
         tw.count[2] += (unsigned)n_cand;
     }
-    if (has == 0u) return true;
-    // candidates, but no sphere penetrates any of them: the chunk's terms are zero, and the
-    // tests' gaps join the clearances
-    if (hits) {
-        if (lane == 0) atomicOr(&sh.hit[(t0 - 1) >> 5], hits << ((t0 - 1) & 31));
-        return false;
-    }
+    if (has == 0u) return kStateZero;
+    // the tests' gaps join the clearances of a half without a penetration
+    if (hits && lane == 0) atomicOr(&sh.hit[(t0 - 1) >> 5], hits << ((t0 - 1) & 31));
     clearance = fminf(clearance, warp_fmin(gap_s));
     clearance_moving = fminf(clearance_moving, warp_fmin(gap_m));
     clearance_top = fminf(clearance_top, warp_fmin(gap_t));
-    return true;
+    return (__any_sync(0xffffffffu, hit_s) ? 0 : kStateZeroStatic) | (__any_sync(0xffffffffu, hit_m) ? 0 : kStateZeroMoving);
+}
+
+// The scale dL/dh of residual r, (lambda_r + mu sqrt(w) h) sqrt(w).
+__device__ __forceinline__ float residual_scale(const TShared& sh, int r, float sqw, float h) {
+    const float hw = sqw * h;
+    return (sh.lam[r] + sh.mu * hw) * sqw;
+}
+
+// C_coll of the placed tower: the fixed-order sum over the slices.
+__device__ __forceinline__ float tower_collisions(const TShared& sh, int n_pu) {
+    float c = 0.f;
+#pragma unroll 1
+    for (int u = 0; u < n_pu; ++u) c += sh.pcu[u][0];
+    return c;
 }
 
 // Residuals of the start group at the grasp (place = false) or place configuration of block b
-// from that configuration's frames: position error, roll and pitch, or roll and pitch, to h_out;
-// the roll and pitch torques to rpt.
-__device__ __forceinline__ void start_residuals(const TrajScalars& sc, int b, bool place, const SpecialFrames& sf,
-                                                float* h_out, float rpt[6]) {
+// from that configuration's frames: position error, roll and pitch, or roll and pitch, to sh.h
+// from r on, their scales to sh.s; the roll and pitch torques to rpt.
+__device__ __forceinline__ void start_residuals(const TrajScalars& sc, TShared& sh, int b, bool place,
+                                                const SpecialFrames& sf, int r0, float rpt[6]) {
     float Rb[9], pb[3];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
@@ -628,20 +651,20 @@ __device__ __forceinline__ void start_residuals(const TrajScalars& sc, int b, bo
     }
     float roll, pitch;
     roll_pitch_torque<float>(Rb, roll, pitch, rpt, rpt + 3);
-    if (!place) {
-        h_out[0] = pb[0] - sc.init[b].x;
-        h_out[1] = pb[1] - sc.init[b].y;
-        h_out[2] = pb[2] - sc.init[b].z;
-        h_out += 3;
+    const float h[5] = {roll, pitch, pb[0] - sc.init[b].x, pb[1] - sc.init[b].y, pb[2] - sc.init[b].z};
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const int r = r0 + (place ? i : (i + 3) % 5);   // grasp: x, y, z, roll, pitch
+        if (place && i >= 2) continue;
+        sh.h[r] = h[i];
+        sh.s[r] = residual_scale(sh, r, sc.sqw[0], h[i]);
     }
-    h_out[0] = roll;
-    h_out[1] = pitch;
 }
 
-// Their weighted joint gradient sum_r s_r dh_r/dq, plus at a place configuration the placed-pose
-// gradient g4 through fk, from the torques the residual pass left in rpt (which may be grad_out).
-__device__ __forceinline__ void start_gradient(bool place, const SpecialFrames& sf, const float* s_r, const float* g4,
-                                               const float rpt[6], float grad_out[7]) {
+// Joint k of their weighted gradient sum_r s_r dh_r/dq, plus at a place configuration the
+// placed-pose gradient g4 through fk, from the torques the residual pass left in rpt.
+__device__ __forceinline__ float start_gradient(bool place, const SpecialFrames& sf, const float* s_r, const float* g4,
+                                                const float rpt[6], int k) {
     float Rb[9], pb[3];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
@@ -666,16 +689,13 @@ __device__ __forceinline__ void start_gradient(bool place, const SpecialFrames& 
     M[0] += pb[1] * F[2] - pb[2] * F[1];
     M[1] += pb[2] * F[0] - pb[0] * F[2];
     M[2] += pb[0] * F[1] - pb[1] * F[0];
-#pragma unroll 1
-    for (int k = 0; k < 7; ++k) {
-        const float2 f0 = sf.Z[k][0], f1 = sf.Z[k][1], f2 = sf.Z[k][2];
-        const float ok[3] = {f0.y, f1.y, f2.y};
-        // z . (M - o x F)
-        const float tx = M[0] - (ok[1] * F[2] - ok[2] * F[1]);
-        const float ty = M[1] - (ok[2] * F[0] - ok[0] * F[2]);
-        const float tz = M[2] - (ok[0] * F[1] - ok[1] * F[0]);
-        grad_out[k] = f0.x * tx + f1.x * ty + f2.x * tz;
-    }
+    const float2 f0 = sf.Z[k][0], f1 = sf.Z[k][1], f2 = sf.Z[k][2];
+    const float ok[3] = {f0.y, f1.y, f2.y};
+    // z . (M - o x F)
+    const float tx = M[0] - (ok[1] * F[2] - ok[2] * F[1]);
+    const float ty = M[1] - (ok[2] * F[0] - ok[0] * F[2]);
+    const float tz = M[2] - (ok[0] * F[1] - ok[1] * F[0]);
+    return f0.x * tx + f1.x * ty + f2.x * tz;
 }
 
 // Collisions of the placed tower (the C_coll residual of the placement terms), slice u of its
@@ -704,8 +724,9 @@ __device__ __forceinline__ void placed_slice(const TrajScalars& sc, const float4
     const float r = h.w;
     const int n_cw = t_cub_words(sc.n_cub), n_w = t_words(sc.n_cub, sc.n_osph);
     const float4* bbox = aabb + 64 * (n_w - 1);
-    // the tower's box
-    const float4 mlo = bbox[2 * (lane & 15)], mhi = bbox[2 * (lane & 15) + 1];   // empty for lanes beyond B
+    // the box of the slice's blocks
+    const int bj = min(4 * u + (lane & 3), B - 1);
+    const float4 mlo = bbox[2 * bj], mhi = bbox[2 * bj + 1];
     const float tlx = warp_fmin(mlo.x), tly = warp_fmin(mlo.y), tlz = warp_fmin(mlo.z);
     const float thx = warp_fmax(mhi.x), thy = warp_fmax(mhi.y), thz = warp_fmax(mhi.z);
     float coll = 0.f, maxpen = 0.f;
@@ -715,21 +736,17 @@ __device__ __forceinline__ void placed_slice(const TrajScalars& sc, const float4
         sh.pgc[u][lane >> 1][2 * (lane & 1) + 1] = 0.f;
         __syncwarp();
     }
-    // the environment's obstacles near the tower, then the blocks below in the stack: a sphere of
-    // j against the cuboids of i < j (the slice's highest block bounds i)
+    // the environment's obstacles and the blocks below that box could touch: a sphere of j against
+    // the cuboids of i < j (the slice's highest block bounds i)
     const int i_end = min(B - 1, (min(32 * u + 31, n_items - 1) >> 3));
 #pragma unroll 1
     for (int wd = 0; wd < n_w; ++wd) {
         const bool blocks = wd == n_w - 1;
         const float4* box = aabb + 64 * wd;
-        unsigned mk;
-        if (blocks) {
-            mk = (1u << i_end) - 1u;
-        } else {
-            const float4 lo = box[2 * lane], hi = box[2 * lane + 1];
-            mk = __ballot_sync(0xffffffffu,
-                               !(lo.x > thx || hi.x < tlx || lo.y > thy || hi.y < tly || lo.z > thz || hi.z < tlz));
-        }
+        const float4 clo = box[2 * lane], chi = box[2 * lane + 1];
+        unsigned mk = __ballot_sync(
+            0xffffffffu, !(clo.x > thx || chi.x < tlx || clo.y > thy || chi.y < tly || clo.z > thz || chi.z < tlz));
+        if (blocks) mk &= (1u << i_end) - 1u;
 #pragma unroll 1
         while (mk) {
             const int bit = __ffs(mk) - 1;
@@ -790,13 +807,23 @@ __device__ __forceinline__ void cuboid_aabb(const float4* c, float4* box) {
     box[1] = make_float4(c[0].x + ex, c[0].y + ey, c[0].z + ez, 0.f);
 }
 
+// The run of configurations [t_lo, t_hi) that warp w of a group steps in traj_step: equal runs over
+// the warps but the first.
+template <int kPpc>
+__device__ __forceinline__ void step_run(int C, int w, int& t_lo, int& t_hi) {
+    const int run = (C + kGrpWarps<kPpc> - 2) / (kGrpWarps<kPpc> - 1);
+    t_lo = w > 0 ? min(C, (w - 1) * run) : C;
+    t_hi = min(C, t_lo + run);
+}
+
 // Evaluate the whole particle: kinematics of the grasp/place configurations and the placed
 // poses, the configuration loop, residuals and objective; with `grad`, the parts of dL/dq that
-// traj_step adds up (the collision groups' rows, the grasp and place rows in sh.extra).
+// traj_step adds up (the collision groups' rows and fixed-point sums, the residuals' scales and
+// the placement gradient without its collision terms).
 template <bool kP2P, int kTile, int kPpc>
 __device__ void traj_evaluate(const TrajScalars& sc, const LaneSpheres& ls, const float4* cub, const float4* osph,
                               float4* aabb, TShared& sh, TWarp* tws, SpecialFrames* sp, float* q, float* rows,
-                              float* disp, float* cblk, __half2* cgap, unsigned char* ccand, float* ctopm,
+                              float* disp, float* cblk, __half2* cgap, unsigned char* state, float* ctopm,
                               __half* ctop, bool grad, bool last) {
     constexpr int kWarps = kGrpWarps<kPpc>;
     const int tid = grp_tid<kPpc>(), lane = tid & 31, w = tid >> 5;
@@ -824,6 +851,15 @@ __device__ void traj_evaluate(const TrajScalars& sc, const LaneSpheres& ls, cons
     if (tid < kMaxC / 32) sh.hit[tid] = 0u;
     if (tid <= kChunk) sh.n_tier[tid] = 0;
     if (tid == 0) { sh.fx_tot[0] = sh.fx_tot[1] = 0; sh.next = 0; }
+    // start residuals: grasp configurations on lanes 0..15, place configurations on 16..31
+    auto start_job = [&]() {
+        const int b = lane & 15;
+        const bool place = lane >= 16;
+        if (b >= B) return;
+        const int r = place ? 5 * B + 2 * b : 5 * b;
+        if (!place || !p2p) start_residuals(sc, sh, b, place, sp[2 * b + place], r, sh.rpt[2 * b + place]);
+        else sh.h[r] = sh.h[r + 1] = 0.f;
+    };
     float acc_max = 0.f;
     bool special = true;
     int gi = w;
@@ -869,30 +905,36 @@ __device__ void traj_evaluate(const TrajScalars& sc, const LaneSpheres& ls, cons
                     }
                     if (lane < B) sh.blk_cum[lane] += moved;
                     if (lane == 0) sh.pose_prev_ok = 1;
+                } else if (w == 1 && !p2p) {
+                    start_job();   // beside the placed poses, which keep warp 0 about as long
                 }
                 grp_sync<kPpc>();
-                // (2) the work queue, in order: the chunks to evaluate, which are those without a valid cached
-                // cull (terms zero at its last cull, and the motion since below its clearances), by tier (4, 3,
-                // 2, 1 configurations with candidates at the last cull, then the chunks to cull again); the
-                // residual jobs (they need only the placed poses and the special frames); the slices of the
-                // placed tower.  The smaller items come last, so that the warps finish together.  Each warp
-                // appends the chunks of its 32-chunk groups to the tiers' lists.
+                // (2) the work queue, in order: the chunks to evaluate, which are those with a half that has no
+                // valid cached cull (terms zero at its last cull, and the motion since below its clearances), by
+                // tier (with a penetration: 4, 3, 2, 1 configurations with candidates; then the others); the
+                // placement residuals (they need only the placed poses); the slices of the placed tower.  The
+                // smaller items come last, so that the warps finish together.  Each warp appends the chunks
+                // of its 32-chunk groups to the tiers' lists.
 #pragma unroll 1
                 for (int gr = w; gr < kChunkGroups; gr += kWarps) {
                     const int chk = 32 * gr + lane;
                     const int t0 = 1 + kChunk * chk, nc = min(kChunk, C - t0);
-                    bool active = chk < n_chunks;
-                    if (active && ccand[chk] == 0) {
+                    int tier = -1;
+                    if (chk < n_chunks) {
                         float d = 0.f;
 #pragma unroll 1
                         for (int i = 0; i < nc; ++i) d = fmaxf(d, disp[t0 + i]);
                         const __half2 cg = cgap[chk];
-                        const int top = chunk_block(t0) - 1;
-                        active = !(d < __low2float(cg) && d + (blk_before(top) - cblk[chk]) < __high2float(cg) &&
-                                   d + (own_motion(top) - ctopm[chk]) < __half2float(ctop[chk]));
+                        const int top = chunk_block(t0) - 1, st = state[chk];
+                        const bool skip_s = (st & kStateZeroStatic) && d < __low2float(cg);
+                        const bool skip_m = (st & kStateZeroMoving) && d + (blk_before(top) - cblk[chk]) < __high2float(cg) &&
+                                            d + (own_motion(top) - ctopm[chk]) < __half2float(ctop[chk]);
+                        if (!(skip_s && skip_m)) {
+                            tier = (st & kStateZero) == kStateZero ? kChunk : kChunk - (st & kStateCand);
+                            state[chk] = (unsigned char)((st & ~(kStateSkipStatic | kStateSkipMoving)) |
+                                                         (skip_s ? kStateSkipStatic : 0) | (skip_m ? kStateSkipMoving : 0));
+                        }
                     }
-                    // tier: kChunk - (configurations with candidates), kChunk for a chunk to cull again
-                    const int tier = active ? (ccand[chk] == 0 ? kChunk : kChunk - ccand[chk]) : -1;
                     unsigned same = 0u;   // lane tr <= kChunk: the group's chunks in tier tr
 #pragma unroll
                     for (int tr = 0; tr <= kChunk; ++tr) {
@@ -929,10 +971,12 @@ __device__ void traj_evaluate(const TrajScalars& sc, const LaneSpheres& ls, cons
                 placed_slice(sc, cub, osph, aabb, sh, grad, idx);
                 continue;
             }
-            if (tier > kChunk && idx == 0) {
-                // placement residuals (tower terms) with their unit-coefficient support factors
+            if (tier > kChunk) {
+                // placement residuals (tower terms) with their unit-coefficient support factors; point to
+                // point, which has none, takes the start residuals here
                 float my_D = 0.f, my_e = 0.f;
-                if (!p2p) place_stack_warp(sc, sh.pose, kPlaceUnit, nullptr, nullptr, nullptr, sh.ps, sh.blk, my_D, my_e);
+                if (p2p) start_job();
+                else place_stack_warp(sc, sh.pose, kPlaceUnit, nullptr, nullptr, nullptr, sh.ps, sh.blk, my_D, my_e);
                 const float c_stable = warp_sum(lane < B ? my_D : 0.f);
                 const float c_height = warp_sum(lane < B ? my_e * my_e : 0.f);
                 const float max_D = warp_fmax(lane < B ? my_D : 0.f);
@@ -940,21 +984,14 @@ __device__ void traj_evaluate(const TrajScalars& sc, const LaneSpheres& ls, cons
                 if (lane < B) {
                     sh.h[7 * B + lane] = my_e;
                     sh.h[8 * B + lane] = my_D;
+                    sh.s[7 * B + lane] = residual_scale(sh, 7 * B + lane, sc.sqw[1], my_e);
+                    sh.s[8 * B + lane] = residual_scale(sh, 8 * B + lane, sc.sqw[2], my_D);
+                }
+                if (grad && !p2p) {   // their part of the placement gradient (the collisions' part follows the queue)
+                    __syncwarp();
+                    place_stack_grad(sc, sh.ps, &sh.s[8 * B], &sh.s[7 * B], sh.inv_above, sh.g4);
                 }
                 if (lane == 0) { sh.c_stable = c_stable; sh.c_height = c_height; sh.pm_D = max_D; sh.pm_dz = max_dz; }
-                continue;
-            }
-            if (tier > kChunk) {
-                // start residuals: grasp configurations on lanes 0..15, place configurations on 16..31
-                const int b = lane & 15;
-                const bool place = lane >= 16;
-                if (b < B) {
-                    if (!place || !p2p)
-                        start_residuals(sc, b, place, sp[2 * b + place], &sh.h[place ? 5 * B + 2 * b : 5 * b],
-                                        sh.extra[place ? B + b : b]);
-                    else
-                        sh.h[5 * B + 2 * b] = sh.h[5 * B + 2 * b + 1] = 0.f;
-                }
                 continue;
             }
             chk = sh.active[tier][idx];
@@ -972,36 +1009,51 @@ __device__ void traj_evaluate(const TrajScalars& sc, const LaneSpheres& ls, cons
         const int t0 = 1 + kChunk * chk, nc = min(kChunk, C - t0), seg_c = div_steps(t_c - 1, inv_S);
         float clearance, clearance_moving, clearance_top, c2[2] = {0.f, 0.f};
         int n_cand;
-        const bool zero = chunk_collisions<kTile>(sc, ls, cub, osph, aabb, sh, tws[w], rows, t0, nc, seg_c, grad, box,
-                                                  c2[0], c2[1], acc_max, n_cand, clearance, clearance_moving,
-                                                  clearance_top);
-        if (!zero) {
+        const int skip = state[chk];
+        const int zero = chunk_collisions<kTile>(sc, ls, cub, osph, aabb, sh, tws[w], rows, t0, nc, seg_c, skip, grad, box,
+                                                 c2[0], c2[1], acc_max, n_cand, clearance, clearance_moving,
+                                                 clearance_top);
+        if (zero != kStateZero) {
             const float v = warp_sums<2>(c2);   // lane 0: the arm's sum, lane 16: the held block's
             if ((lane & 15) == 0) fx_add(&sh.fx_tot[lane >> 4], v);
         }
+        const float d = warp_fmax(lane < nc ? disp[t0 + lane] : 0.f);
         if (lane == 0) {
-            ccand[chk] = zero ? 0 : (unsigned char)n_cand;   // 0: a chunk whose terms are zero (cacheable)
+            state[chk] = (unsigned char)(n_cand | zero);
+            const __half2 cg = cgap[chk];
             const int top = chunk_block(t0) - 1;
-            cblk[chk] = blk_before(top);
-            ctopm[chk] = own_motion(top);
+            // a skipped half keeps its clearance less the motion so far (disp starts at zero again) and the
+            // blocks' motions it was taken at
+            float cs = clearance - kClearSlack, cm = clearance_moving - kClearSlack, ct = clearance_top - kClearSlack;
+            if (skip & kStateSkipStatic) cs = __fsub_rd(__low2float(cg), d);
+            if (skip & kStateSkipMoving) {
+                cm = __fsub_rd(__high2float(cg), d);
+                ct = __fsub_rd(__half2float(ctop[chk]), d);
+            } else {
+                cblk[chk] = blk_before(top);
+                ctopm[chk] = own_motion(top);
+            }
             // fp16, rounded down: still lower bounds on the clearances
-            cgap[chk] = __halves2half2(__float2half_rd(clearance - kClearSlack),
-                                       __float2half_rd(clearance_moving - kClearSlack));
-            ctop[chk] = __float2half_rd(clearance_top - kClearSlack);
+            cgap[chk] = __halves2half2(__float2half_rd(cs), __float2half_rd(cm));
+            ctop[chk] = __float2half_rd(ct);
         }
+        __syncwarp();
         if (lane < nc) disp[t0 + lane] = 0.f;
         __syncwarp();
     }
     acc_max = warp_fmax(acc_max);
     if (lane == 0) tws[w].maxpen = acc_max;
+    int t_lo, t_hi;
+    step_run<kPpc>(C, w, t_lo, t_hi);
+    if (lane < 4 && t_lo < t_hi)   // for the step: the run's first row, then its last
+        tws[w].edge[lane >> 1][lane & 1] = reinterpret_cast<const float4*>(q + 8 * (lane < 2 ? t_lo : t_hi - 1))[lane & 1];
     grp_sync<kPpc>();
 
-    // (3) warp 0: the group sums, then the objective and dL/dh
+    if (!last) return;
+
+    // (3) warp 0, after the last evaluation: the objective and the metrics
     if (w == 0) {
-        const float tot_a = fx_value(sh.fx_tot[0]), tot_b = fx_value(sh.fx_tot[1]);
-        float c_coll = 0.f;   // fixed-order sum over the slices
-#pragma unroll 1
-        for (int u = 0; u < n_pu; ++u) c_coll += sh.pcu[u][0];
+        const float tot_a = fx_value(sh.fx_tot[0]), tot_b = fx_value(sh.fx_tot[1]), c_coll = tower_collisions(sh, n_pu);
         if (lane == 0) {
             sh.h[9 * B] = c_coll;
             sh.h[9 * B + 1] = tot_a;
@@ -1011,83 +1063,71 @@ __device__ void traj_evaluate(const TrajScalars& sc, const LaneSpheres& ls, cons
         float Lp = 0.f;
 #pragma unroll 1
         for (int r = lane; r < NR; r += 32) {
-            const float sw = residual_sqrt_weight(sc, r), hw = sw * sh.h[r];
+            const float hw = residual_sqrt_weight(sc, r) * sh.h[r];
             Lp += sh.lam[r] * hw + 0.5f * sh.mu * hw * hw;
-            sh.s[r] = (sh.lam[r] + sh.mu * hw) * sw;
         }
-        __syncwarp();   // sh.s[] was written by other lanes: order those stores before lane 0 reads them
-        if (lane == 0) { sh.s_arm = sh.s[9 * B + 1]; sh.s_blk = sh.s[9 * B + 2]; }
-        if (last) {   // the objective and the metrics, which a descent reads after its last evaluation only
-            const float cm = warp_fmax(lane < kWarps ? tws[lane].maxpen : 0.f);
-            const float pm = warp_fmax(lane < n_pu ? sh.pcu[lane][1] : 0.f);
-            float v_start = 0.f, v_tilt = 0.f;
-            if (lane < B) {
-                const float* hg = &sh.h[5 * lane];
-                const float* hp = &sh.h[5 * B + 2 * lane];
-                v_start = hg[0] * hg[0] + hg[1] * hg[1] + hg[2] * hg[2] + hg[3] * hg[3] + hg[4] * hg[4];
-                v_tilt = hp[0] * hp[0] + hp[1] * hp[1];
-            }
-            const float c_start = warp_sum(v_start + v_tilt);
-            const float m_start = warp_fmax(v_start), m_tilt = warp_fmax(v_tilt);
-            Lp = warp_sum(Lp);
-            if (lane == 0) {
-                sh.c_arm = tot_a; sh.c_blk = tot_b; sh.maxpen = cm;
-                sh.c_coll = c_coll; sh.pm_pen = pm;
-                sh.L = Lp; sh.c_start = c_start; sh.max_start = m_start; sh.max_tilt = m_tilt;
-            }
+        const float cm = warp_fmax(lane < kWarps ? tws[lane].maxpen : 0.f);
+        const float pm = warp_fmax(lane < n_pu ? sh.pcu[lane][1] : 0.f);
+        float v_start = 0.f, v_tilt = 0.f;
+        if (lane < B) {
+            const float* hg = &sh.h[5 * lane];
+            const float* hp = &sh.h[5 * B + 2 * lane];
+            v_start = hg[0] * hg[0] + hg[1] * hg[1] + hg[2] * hg[2] + hg[3] * hg[3] + hg[4] * hg[4];
+            v_tilt = hp[0] * hp[0] + hp[1] * hp[1];
+        }
+        const float c_start = warp_sum(v_start + v_tilt);
+        const float m_start = warp_fmax(v_start), m_tilt = warp_fmax(v_tilt);
+        Lp = warp_sum(Lp);
+        if (lane == 0) {
+            sh.c_arm = tot_a; sh.c_blk = tot_b; sh.maxpen = cm;
+            sh.c_coll = c_coll; sh.pm_pen = pm;
+            sh.L = Lp; sh.c_start = c_start; sh.max_start = m_start; sh.max_tilt = m_tilt;
         }
     }
     grp_sync<kPpc>();
-    if (grad) {
-        // (4) warp 0: placement gradient w.r.t. the placed poses, then the gradient rows of the grasp
-        // (lanes 0..15) and place configurations
-        if (w == 0) {
-            if (!p2p) {
-                place_stack_grad(sc, sh.ps, &sh.s[8 * B], &sh.s[7 * B], sh.g4);
-                const float s_arm = sh.s_arm, s_blk = sh.s_blk, s_coll = sh.s[9 * B];
-#pragma unroll 1
-                for (int i = lane; i < 4 * B; i += 32) {
-                    const int kb = i >> 2, c = i & 3;
-                    const float wa = fx_value(sh.fx_wr[0][kb][c]), wb = fx_value(sh.fx_wr[1][kb][c]);
-                    float gc = sh.pg[kb][c];
-                    if (kb + 1 < B)
-#pragma unroll 1
-                        for (int u = 0; u < n_pu; ++u) gc += sh.pgc[u][kb][c];
-                    sh.g4[i] += s_coll * gc + s_arm * wa + s_blk * wb;
-                }
-                __syncwarp();
-            }
-            const int b = lane & 15;
-            const bool place = lane >= 16;
-            if (b < B && !(place && p2p)) {
-                float* row = sh.extra[place ? B + b : b];
-                start_gradient(place, sp[2 * b + place], &sh.s[place ? 5 * B + 2 * b : 5 * b], &sh.g4[4 * b], row, row);
-            }
-        }
-        grp_sync<kPpc>();
-    }
 }
 
 // One descent step, q <- clamp(q - eta g), and the bound on how far each configuration's spheres
 // moved (disp); or, when grad_out is given, the gradient itself (8 floats per configuration, the
 // last and the fixed first configuration's zero).  The gradient of configuration t: the path term
-// from its neighbours, the joint limits, the collision groups' rows and the grasp or place row.
-// In place, a configuration per lane (rows as float4 pairs): each warp of the group takes a
-// contiguous run of configurations, 32 at a time in ascending order; a row that its neighbour
-// reads after the step is kept in TWarp::edge as it was (the run's first and last rows, and the last
-// row of the previous 32).
+// from its neighbours, the joint limits, the collision groups' rows and, at the grasp and place
+// configurations, their own row.
+// Warp 0 first completes the placement gradient, which only the place configurations' rows need;
+// the other warps step the configurations in between meanwhile and leave the special ones, whose
+// gradient so far goes to sh.partial; after a barrier, a lane per joint adds the special rows
+// and steps those.  (Rows first, then one pass over every configuration: 12 of an evaluation's
+// 41 thousand cycles on the 10-block tower, with one warp at work for 8 of them.)
+// In place, a configuration per lane (rows as float4 pairs): each warp takes a contiguous run of
+// configurations, 32 at a time in ascending order; a row that its neighbour reads after the
+// step is kept in TWarp::edge as it was (the run's first and last rows, kept by traj_evaluate,
+// and the last row of the previous 32).
 // `limits`: joints may lie outside their limits (a step clamps them, so only before the first).
-template <int kPpc>
-__device__ __forceinline__ void traj_step(const TrajScalars& sc, TShared& sh, TWarp* tws, float* q, const float* rows, float* disp,
-                                          float eta, bool limits, float* grad_out) {
+template <bool kP2P, int kPpc>
+__device__ __forceinline__ void traj_step(const TrajScalars& sc, TShared& sh, TWarp* tws, const SpecialFrames* sp, float* q,
+                                          const float* rows, float* disp, float eta, bool limits, float* grad_out) {
     constexpr int kWarps = kGrpWarps<kPpc>;
     const int tid = grp_tid<kPpc>(), lane = tid & 31, w = tid >> 5;
-    const int C = sc.C, S = sc.S;
-    const int run = (C + kWarps - 1) / kWarps, t_lo = min(C, w * run), t_hi = min(C, t_lo + run);
-    if (lane < 4 && t_lo < t_hi)   // the run's first row, then its last
-        tws[w].edge[lane >> 1][lane & 1] = reinterpret_cast<const float4*>(q + 8 * (lane < 2 ? t_lo : t_hi - 1))[lane & 1];
-    grp_sync<kPpc>();
-    const float s_arm = sh.s_arm, s_blk = sh.s_blk, inv_S = sh.inv_S, w2 = 2.f * sc.w_path;
+    const int B = sc.B, C = sc.C, S = sc.S, n_pu = kP2P ? 0 : (8 * B + 31) / 32;
+    int t_lo, t_hi;
+    step_run<kPpc>(C, w, t_lo, t_hi);
+    const float tot_a = fx_value(sh.fx_tot[0]), tot_b = fx_value(sh.fx_tot[1]);
+    const float s_arm = residual_scale(sh, 9 * B + 1, sc.sqw[4], tot_a);
+    const float s_blk = residual_scale(sh, 9 * B + 2, sc.sqw[5], tot_b);
+    if (w == 0) {
+        const float c_coll = tower_collisions(sh, n_pu), s_coll = residual_scale(sh, 9 * B, sc.sqw[3], c_coll);
+        if (lane == 0) { sh.h[9 * B] = c_coll; sh.h[9 * B + 1] = tot_a; sh.h[9 * B + 2] = tot_b; }
+#pragma unroll 1
+        for (int i = lane; i < (kP2P ? 0 : 4 * B); i += 32) {
+            const int kb = i >> 2, c = i & 3;
+            const float wa = fx_value(sh.fx_wr[0][kb][c]), wb = fx_value(sh.fx_wr[1][kb][c]);
+            float gc = sh.pg[kb][c];
+            if (kb + 1 < B)
+#pragma unroll 1
+                for (int u = 0; u < n_pu; ++u) gc += sh.pgc[u][kb][c];
+            sh.g4[i] += s_coll * gc + s_arm * wa + s_blk * wb;
+        }
+    }
+    const float inv_S = sh.inv_S, w2 = 2.f * sc.w_path;
     // a row without collision terms adds s_arm 0 + s_blk 0, which is zero unless a scale is not finite
     const bool all_rows = !(s_arm * 0.f + s_blk * 0.f == 0.f);
 #pragma unroll 1
@@ -1095,7 +1135,7 @@ __device__ __forceinline__ void traj_step(const TrajScalars& sc, TShared& sh, TW
         const int t = t0 + lane;
         const bool in = t < t_hi;
         const float4* qv = reinterpret_cast<const float4*>(q + 8 * min(t, t_hi - 1));
-        const float4* pr = lane > 0 ? qv - 2 : t0 > t_lo ? tws[w].edge[2] : w > 0 ? tws[w - 1].edge[1] : qv;
+        const float4* pr = lane > 0 ? qv - 2 : t0 > t_lo ? tws[w].edge[2] : w > 1 ? tws[w - 1].edge[1] : qv;
         const float4* nx = t + 1 >= C ? qv : t + 1 < t_hi ? qv + 2 : tws[w + 1].edge[0];
         const float4 a0 = qv[0], a1 = qv[1], p0 = pr[0], p1 = pr[1], n0 = nx[0], n1 = nx[1];
         const float v[7] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z};
@@ -1129,14 +1169,11 @@ __device__ __forceinline__ void traj_step(const TrajScalars& sc, TShared& sh, TW
             for (int j = 0; j < 7; ++j) g[j] += s_arm * ga[j] + s_blk * gb[j];
         }
         const int e = div_steps(t, inv_S) - 1;
-        if (in && t > 0 && t == (e + 1) * S) {   // grasp of block e/2 (e even) or place (e odd)
-            const float4* ev = reinterpret_cast<const float4*>(sh.extra[(e & 1 ? sc.B : 0) + (e >> 1)]);
-            const float4 e0 = ev[0], e1 = ev[1];
-            const float ex[7] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z};
-#pragma unroll
-            for (int j = 0; j < 7; ++j) g[j] += ex[j];
-        }
-        if (grad_out) {
+        const bool special = e >= 0 && t == (e + 1) * S;
+        if (in && special) {   // grasp of block e / 2 (e even) or place (e odd)
+            sh.partial[e][0] = make_float4(g[0], g[1], g[2], g[3]);
+            sh.partial[e][1] = make_float4(g[4], g[5], g[6], 0.f);
+        } else if (grad_out) {
             float* go = grad_out + (size_t)t * 8;
             if (t == 0) {
 #pragma unroll
@@ -1164,6 +1201,33 @@ __device__ __forceinline__ void traj_step(const TrajScalars& sc, TShared& sh, TW
             disp[t] += moved * 1.0001f + 1e-7f;
         }
         __syncwarp();   // tws[w].edge[2] before lane 0 reads it
+    }
+    grp_sync<kPpc>();
+    // the special configurations, four per warp: lane 8 c + j, joint j
+    const int n_sp = kP2P ? 1 : 2 * B, j = lane & 7, jj = min(j, 6);
+#pragma unroll 1
+    for (int e = 4 * w + (lane >> 3); e - (lane >> 3) < n_sp; e += 4 * kWarps) {
+        const int b = e >> 1, t = (e + 1) * S;
+        const bool in = e < n_sp && j < 7, place = e & 1;
+        float g = 0.f, moved = 0.f;
+        if (in) {
+            g = reinterpret_cast<const float*>(sh.partial[e])[j];
+            g += start_gradient(place, sp[e], &sh.s[place ? 5 * B + 2 * b : 5 * b], &sh.g4[4 * b], sh.rpt[e], j);
+        }
+        if (grad_out) {
+            if (e < n_sp) grad_out[(size_t)t * 8 + j] = g;
+            continue;
+        }
+        if (in) {
+            const float v = q[8 * t + j], x = v - eta * g;
+            const float nw = fminf(fmaxf(x, sc.qlo[jj]), sc.qhi[jj]);
+            q[8 * t + j] = nw;
+            moved = fabsf(nw - v) * sc.sweep[jj];
+        }
+        moved += __shfl_xor_sync(0xffffffffu, moved, 1);
+        moved += __shfl_xor_sync(0xffffffffu, moved, 2);
+        moved += __shfl_xor_sync(0xffffffffu, moved, 4);
+        if (e < n_sp && j == 0) disp[t] += moved * 1.0001f + 1e-7f;
     }
 }
 
@@ -1246,6 +1310,7 @@ __device__ __forceinline__ void traj_setup(const TrajScalars& sc, unsigned char*
         }
     }
     if (tid == 0) sh.inv_S = 1.f / (float)sc.S;
+    if (tid < kMaxB) sh.inv_above[tid] = tid + 1 < sc.B ? 1.f / (float)(sc.B - 1 - tid) : 0.f;
     if (tid < 8) {
         sh.dh[tid] = tid < 7 ? make_float4(sc.ca[tid], sc.sa[tid], sc.a[tid], sc.d[tid]) : make_float4(1.f, 0.f, 0.f, 0.f);
         sh.th0[tid] = tid < 7 ? sc.th0[tid] : 0.f;
@@ -1274,14 +1339,14 @@ __device__ __forceinline__ void traj_particle(const TrajScalars& sc, const LaneS
     __half2* cgap = reinterpret_cast<__half2*>(cblk + n_chunks);   // (static, moving) clearances
     float* ctopm = reinterpret_cast<float*>(cgap + n_chunks);    // the top block's own motion at the cull
     __half* ctop = reinterpret_cast<__half*>(ctopm + n_chunks);  // clearance to the top block
-    unsigned char* ccand = reinterpret_cast<unsigned char*>(ctop + n_chunks);
+    unsigned char* state = reinterpret_cast<unsigned char*>(ctop + n_chunks);
     const int tid = grp_tid<kPpc>();
     const int C = sc.C, NR = sc.NR;
 #pragma unroll 1
     for (int i = tid; i < C; i += kThreads) disp[i] = 0.f;
 #pragma unroll 1
     for (int i = tid; i < n_chunks; i += kThreads) {
-        cblk[i] = 0.f; cgap[i] = __float2half2_rn(0.f); ccand[i] = kChunk; ctopm[i] = 0.f; ctop[i] = __float2half_rn(0.f);
+        cblk[i] = 0.f; cgap[i] = __float2half2_rn(0.f); state[i] = kChunk; ctopm[i] = 0.f; ctop[i] = __float2half_rn(0.f);
     }
     if (tid < kMaxB) { sh.blk_cum[tid] = 0.f; sh.bown[tid] = 0.f; }
     if (tid == 0) sh.pose_prev_ok = 0;
@@ -1307,10 +1372,10 @@ __device__ __forceinline__ void traj_particle(const TrajScalars& sc, const LaneS
     const int K = mode == kTrajDescend ? io.k_steps : 0;
     for (int k = 1;; ++k) {
         const bool last = k > K;
-        traj_evaluate<kP2P, kTile, kPpc>(sc, ls, cub, osph, aabb, sh, tws, sp, q, rows, disp, cblk, cgap, ccand, ctopm, ctop,
+        traj_evaluate<kP2P, kTile, kPpc>(sc, ls, cub, osph, aabb, sh, tws, sp, q, rows, disp, cblk, cgap, state, ctopm, ctop,
                                          last ? want_grad : true, last);
         if (!last || want_grad)
-            traj_step<kPpc>(sc, sh, tws, q, rows, disp, sc.eta_traj * (1.f - (float)k / (float)K),
+            traj_step<kP2P, kPpc>(sc, sh, tws, sp, q, rows, disp, sc.eta_traj * (1.f - (float)k / (float)K),
                             last || k == 1 || !(sc.w_jl * 0.f == 0.f), last ? grad_out : nullptr);
         if (last) break;
         if (sc.K_al > 0 && k % sc.K_al == 0) {

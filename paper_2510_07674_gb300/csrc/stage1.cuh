@@ -88,8 +88,9 @@ __device__ __forceinline__ void place_stack_warp(const TrajScalars& sc, const fl
 
 // The gradient place_stack_warp writes in mode kPlaceExplicit, from the factors its kPlaceUnit
 // pass left in ps (a_i dD_i/d... = a_i times the unit factor, in the same order of operations).
+// inv_above[k] = 1 / (B - 1 - k), the blocks above block k < B - 1.
 __device__ __forceinline__ void place_stack_grad(const TrajScalars& sc, const StackScratch& ps, const float* a_in,
-                                                 const float* b_in, float* g) {
+                                                 const float* b_in, const float* inv_above, float* g) {
     const int lane = threadIdx.x & 31;
     const int B = sc.B;
     if (lane < B) {
@@ -97,7 +98,7 @@ __device__ __forceinline__ void place_stack_grad(const TrajScalars& sc, const St
         float gx = -(a_in[i] * ps.stab[i][0]), gy = -(a_in[i] * ps.stab[i][1]);
 #pragma unroll 1
         for (int k = 0; k < i; ++k) {
-            const float inv = 1.f / (float)(B - 1 - k);
+            const float inv = inv_above[k];
             gx += (a_in[k] * ps.stab[k][0]) * inv;
             gy += (a_in[k] * ps.stab[k][1]) * inv;
         }
