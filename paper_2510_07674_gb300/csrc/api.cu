@@ -137,7 +137,7 @@ static void for_each_buffer(spasm_problem* pr, int B, int C, int n_cub, int n_os
     f(pr->d_sc, 1);
     f(pr->d_chkacc, P);
     f(pr->d_ctl, 1);
-    f(pr->d_rows, (size_t)kTrajSlots * C * 16);
+    f(pr->d_rows, (size_t)traj_slots(B, C, n_cub, n_osph) * C * 16);
     f(pr->d_work, 1);
 }
 
@@ -398,7 +398,7 @@ static spasm_status create_problem_impl(const spasm_robot* robot, const spasm_ob
     }
     pr->stats.h2d_bytes += (long long)(cub.size() * sizeof(float4) + osph.size() * sizeof(float4) +
                                        cub64.size() * sizeof(double) + osph64.size() * sizeof(double));
-    const size_t need = traj_cta_smem_bytes(sc, 1);
+    const size_t need = traj_cta_smem_bytes(sc, 1, false);
     int dev = 0, max_smem = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -658,7 +658,7 @@ extern "C" spasm_status spasm_set_kernel_config(spasm_problem_t pr, const spasm_
     int dev = 0, max_smem = 0;
     SPASM_CUDA(cudaGetDevice(&dev));
     SPASM_CUDA(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    if (traj_cta_smem_bytes(pr->sc, cfg->particles_per_cta) > (size_t)max_smem)
+    if (traj_cta_smem_bytes(pr->sc, cfg->particles_per_cta, true) > (size_t)max_smem)
         return fail(SPASM_ERR_INVALID, "the shared memory of that many particles per CTA does not fit this problem");
     SPASM_TRY(finalize(pr));
     SPASM_TRY(host_wait(pr));
@@ -673,8 +673,9 @@ extern "C" spasm_status spasm_set_kernel_config(spasm_problem_t pr, const spasm_
 extern "C" spasm_status spasm_traj_residency(spasm_problem_t pr, int* single, int* batched) {
     if (!pr || !single || !batched) return fail(SPASM_ERR_INVALID, "null argument");
     *single = traj_ctas_per_sm(pr->sc);
-    const int ppc = traj_ppc(pr->sc, pr->sc.Q);
-    *batched = traj_batch_ctas_per_sm(traj_cta_smem_bytes(pr->sc, ppc), pr->sc.sphere_tiling, ppc);
+    const size_t two = traj_cta_smem_bytes(pr->sc, 2, true) + kBatchStaticSmem;
+    const int ppc = pr->sc.particles_per_cta ? pr->sc.particles_per_cta : traj_auto_ppc(two, 0, pr->sc.Q, pr->sc.B, pr->sc.C);
+    *batched = traj_batch_ctas_per_sm(traj_cta_smem_bytes(pr->sc, ppc, true), pr->sc.sphere_tiling, ppc);
     return SPASM_OK;
 }
 

@@ -137,10 +137,10 @@ JobList make_jobs(spasm_problem_t* prs, const std::vector<int>& live, int per_fe
         int blocks = 0;
         for (int i : live) {
             blocks = std::max(blocks, prs[i]->sc.B);
-            two = std::max(two, traj_cta_smem_bytes(prs[i]->sc, 2) + kBatchStaticSmem);
+            two = std::max(two, traj_cta_smem_bytes(prs[i]->sc, 2, true) + kBatchStaticSmem);
             particles += prs[i]->sc.Q;
         }
-        ppc = traj_auto_ppc(two, particles, blocks);
+        ppc = traj_auto_ppc(two, 0, particles, blocks, 0);
     }
     L.ppc = ppc;
     for (int i : live) {
@@ -161,7 +161,7 @@ JobList make_jobs(spasm_problem_t* prs, const std::vector<int>& live, int per_fe
         j.n = pr->sc.Q;
         j.first = L.n_items;
         L.n_items += (pr->sc.Q + per_fetch - 1) / per_fetch;
-        L.cta_bytes = std::max(L.cta_bytes, traj_cta_smem_bytes(pr->sc, ppc));
+        L.cta_bytes = std::max(L.cta_bytes, traj_cta_smem_bytes(pr->sc, ppc, true));
         L.jobs.push_back(j);
     }
     return L;

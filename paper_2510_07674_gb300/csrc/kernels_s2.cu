@@ -18,15 +18,14 @@ constexpr int kSlots = 2;   // sphere items per lane: up to 56 robot + 8 held-bl
 
 constexpr int kChunk = 4;   // configurations whose kinematics one warp evaluates together
 
-// A trajectory CTA of 8 warps runs 1 or 2 particles at once (particles per CTA, a launch
-// option): each on its own group of 8 or 4 warps, with its own region of dynamic shared memory
-// and its own named barrier 1 + group.  With one particle the group is the whole CTA.
-// Two particles of 4 warps are the shape for full launches: an evaluation has a serial chain of
-// phases that keep one or two warps busy (grasp and place frames, placed poses, objective,
-// gradient rows), about 20k of its 70k cycles, and with two CTAs of 8 warps per SM (the
-// registers' limit) four particles overlap those chains instead of two.  One particle of 8
-// warps finishes a single particle sooner, so it takes launches that would not fill the SMs
-// otherwise (traj_auto_ppc).
+// A trajectory CTA of 8 warps runs 1, 2 or 4 particles at once: each on its own group of 8, 4 or
+// 2 warps, with its own region of dynamic shared memory and its own named barrier 1 + group.
+// With one particle the group is the whole CTA.  An evaluation has a serial chain of phases that
+// keep one or two warps busy (grasp and place frames, placed poses, placement gradient) and a
+// queue of a dozen coarse items, so the fewer warps a particle has the less they wait for one
+// another; two CTAs per SM (the registers' limit) overlap 2, 4 or 8 particles' chains.  One
+// particle of 8 warps finishes sooner, so it takes launches that would not fill the SMs
+// otherwise; the rule is traj_auto_ppc's.
 template <int kPpc>
 constexpr int kGrpWarps = kTWarps / kPpc;
 template <int kPpc>
@@ -38,8 +37,7 @@ __device__ __forceinline__ int grp_index() { return kPpc == 1 ? 0 : (int)(thread
 template <int kPpc>
 __device__ __forceinline__ void grp_sync() {
     if (kPpc == 1) __syncthreads();
-    else if (threadIdx.x < kGrpThreads<kPpc>) asm volatile("bar.sync 1, %0;" ::"n"(kGrpThreads<kPpc>) : "memory");
-    else asm volatile("bar.sync 2, %0;" ::"n"(kGrpThreads<kPpc>) : "memory");
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + grp_index<kPpc>()), "n"(kGrpThreads<kPpc>) : "memory");
 }
 
 // Cached cull.  When no sphere of a chunk penetrates a static obstacle (the environment, blocks
@@ -102,6 +100,7 @@ struct SpecialFrames {
 
 struct TShared {
     float4 blk[2 * kMaxB][4];   // block cuboids: k placed this iteration, 16 + k at the initial pose
+    float4 bbox[2 * kMaxB][2];  // their axis-aligned boxes (lo, hi): the word of blocks
     float pose[4 * kMaxB];   // placed poses (x, y, z, yaw)
     float g4[4 * kMaxB];     // dL/d(placed pose)
     float h[kMaxNR], lam[kMaxNR], s[kMaxNR];
@@ -137,37 +136,43 @@ struct TShared {
     int particle;                 // the particle the group works on
 };
 
+// The environment of a problem: barrier words, cuboids, spheres, their boxes.
 __host__ __device__ inline size_t t_env_offset() { return 16; }
 __host__ __device__ inline size_t t_aabb_offset(int n_cub, int n_osph) {
     return (16 + (size_t)n_cub * 64 + (size_t)n_osph * 16 + 15) & ~(size_t)15;
 }
-__host__ __device__ inline size_t t_shared_offset(int n_cub, int n_osph) {
-    return t_aabb_offset(n_cub, n_osph) + (size_t)t_words(n_cub, n_osph) * 32 * 32;
+__host__ __device__ inline size_t t_env_bytes(int n_cub, int n_osph) {
+    return (t_aabb_offset(n_cub, n_osph) + (size_t)(t_words(n_cub, n_osph) - 1) * 32 * 32 + 127) & ~(size_t)127;
 }
-__host__ __device__ inline size_t t_warp_offset(int n_cub, int n_osph) {
-    return (t_shared_offset(n_cub, n_osph) + sizeof(TShared) + 15) & ~(size_t)15;
-}
-__host__ __device__ inline size_t t_q_offset(int n_cub, int n_osph, int warps) {
-    return t_warp_offset(n_cub, n_osph) + (size_t)warps * sizeof(TWarp);
-}
-__host__ __device__ inline size_t t_sp_offset(int n_cub, int n_osph, int C, int warps) {
-    return t_q_offset(n_cub, n_osph, warps) + (size_t)C * 8 * sizeof(float);
-}
+// The region of a particle group.
+__host__ __device__ inline size_t t_warp_offset() { return (sizeof(TShared) + 15) & ~(size_t)15; }
+__host__ __device__ inline size_t t_q_offset(int warps) { return t_warp_offset() + (size_t)warps * sizeof(TWarp); }
+__host__ __device__ inline size_t t_sp_offset(int C, int warps) { return t_q_offset(warps) + (size_t)C * 8 * sizeof(float); }
 __host__ __device__ inline int t_n_chunks(int C) { return (C - 1 + kChunk - 1) / kChunk; }
 // cached cull state: per configuration the motion bound since its chunk's last cull; per
 // chunk, at that cull, the motion bound of the placed blocks below its top block and the top
 // block's own motion, its (static, moving) clearances as an fp16 pair, its fp16 clearance to
 // the top block and its state (kState*)
-__host__ __device__ inline size_t t_cache_offset(int n_cub, int n_osph, int C, int B, int warps) {
-    return (t_sp_offset(n_cub, n_osph, C, warps) + (size_t)2 * B * sizeof(SpecialFrames) + 15) & ~(size_t)15;
+__host__ __device__ inline size_t t_cache_offset(int C, int B, int warps) {
+    return (t_sp_offset(C, warps) + (size_t)2 * B * sizeof(SpecialFrames) + 15) & ~(size_t)15;
 }
-// Shared memory of one particle's group.  The gradient rows of the collision groups are not in
+// Shared memory of one particle's group, rounded to 128 bytes.  The gradient rows of the collision groups are not in
 // it: only the chunks with a penetration have any (4 of 155 per evaluation on the 10-block
 // tower), so they go to the launch's scratch in global memory (TrajIO::rows), which stays in L2;
 // two row buffers here would cost 40 of the region's then 95 KB.
-size_t traj_smem_bytes(const TrajScalars& sc, int ppc) {
-    return t_cache_offset(sc.n_cub, sc.n_osph, sc.C, sc.B, kTWarps / ppc) + (size_t)sc.C * sizeof(float) +
-           (size_t)t_n_chunks(sc.C) * (3 * sizeof(float) + sizeof(__half) + sizeof(unsigned char));
+static size_t t_region(int C, int B, int ppc) {
+    return (t_cache_offset(C, B, kTWarps / ppc) + (size_t)C * sizeof(float) +
+            (size_t)t_n_chunks(C) * (3 * sizeof(float) + sizeof(__half) + sizeof(unsigned char)) + 127) &
+           ~(size_t)127;
+}
+
+size_t traj_cta_smem_bytes(const TrajScalars& sc, int ppc, bool batched) {
+    const size_t env = t_env_bytes(sc.n_cub, sc.n_osph);
+    return (batched ? ppc : 1) * env + ppc * t_region(sc.C, sc.B, ppc);
+}
+
+int traj_slots(int B, int C, int n_cub, int n_osph) {
+    return t_env_bytes(n_cub, n_osph) + 4 * t_region(C, B, 4) <= kHalfSmem ? 2 * kTrajSlots : kTrajSlots;
 }
 
 // Sphere item held in slot k by a lane: strided tiling, item lane + 32 k (the spheres of a link
@@ -414,7 +419,7 @@ __device__ __forceinline__ int chunk_collisions(const TrajScalars& sc, const Lan
 #pragma unroll 1
     for (int wd = wd0; wd < n_w; ++wd) {
         const bool blocks = wd == n_w - 1;
-        const float4* box = aabb + 64 * wd;
+        const float4* box = blocks ? sh.bbox[0] : aabb + 64 * wd;
         const float4 clo = box[2 * lane], chi = box[2 * lane + 1];
         const float s1 = fmaxf(fmaxf(fmaxf(clo.x - hi_x, lo_x - chi.x), fmaxf(clo.y - hi_y, lo_y - chi.y)),
                                fmaxf(clo.z - hi_z, lo_z - chi.z));
@@ -460,7 +465,7 @@ __device__ __forceinline__ int chunk_collisions(const TrajScalars& sc, const Lan
         // the top block: the gap from each link box of the configurations it concerns
         float ct = 3.4e38f;
         if (top >= 0 && top < b_lane) {
-            const float4 blo = aabb[64 * (n_w - 1) + 2 * top], bhi = aabb[64 * (n_w - 1) + 2 * top + 1];
+            const float4 blo = sh.bbox[top][0], bhi = sh.bbox[top][1];
             const float g = fmaxf(fmaxf(fmaxf(blo.x - lb[3], lb[0] - bhi.x), fmaxf(blo.y - lb[4], lb[1] - bhi.y)),
                                   fmaxf(blo.z - lb[5], lb[2] - bhi.z));
             if (g > 0.f) ct = g;   // an overlapping box is tested against the spheres, which give the gap
@@ -723,10 +728,9 @@ __device__ __forceinline__ void placed_slice(const TrajScalars& sc, const float4
     const float cz = sh.pose[4 * j + 2] + lz;
     const float r = h.w;
     const int n_cw = t_cub_words(sc.n_cub), n_w = t_words(sc.n_cub, sc.n_osph);
-    const float4* bbox = aabb + 64 * (n_w - 1);
     // the box of the slice's blocks
     const int bj = min(4 * u + (lane & 3), B - 1);
-    const float4 mlo = bbox[2 * bj], mhi = bbox[2 * bj + 1];
+    const float4 mlo = sh.bbox[bj][0], mhi = sh.bbox[bj][1];
     const float tlx = warp_fmin(mlo.x), tly = warp_fmin(mlo.y), tlz = warp_fmin(mlo.z);
     const float thx = warp_fmax(mhi.x), thy = warp_fmax(mhi.y), thz = warp_fmax(mhi.z);
     float coll = 0.f, maxpen = 0.f;
@@ -742,7 +746,7 @@ __device__ __forceinline__ void placed_slice(const TrajScalars& sc, const float4
 #pragma unroll 1
     for (int wd = 0; wd < n_w; ++wd) {
         const bool blocks = wd == n_w - 1;
-        const float4* box = aabb + 64 * wd;
+        const float4* box = blocks ? sh.bbox[0] : aabb + 64 * wd;
         const float4 clo = box[2 * lane], chi = box[2 * lane + 1];
         unsigned mk = __ballot_sync(
             0xffffffffu, !(clo.x > thx || chi.x < tlx || clo.y > thy || chi.y < tly || clo.z > thz || chi.z < tlz));
@@ -807,13 +811,22 @@ __device__ __forceinline__ void cuboid_aabb(const float4* c, float4* box) {
     box[1] = make_float4(c[0].x + ex, c[0].y + ey, c[0].z + ez, 0.f);
 }
 
-// The run of configurations [t_lo, t_hi) that warp w of a group steps in traj_step: equal runs over
-// the warps but the first.
-template <int kPpc>
+// An empty box: never a candidate.
+__device__ __forceinline__ void empty_box(float4* box) {
+    box[0] = make_float4(3.4e38f, 3.4e38f, 3.4e38f, 0.f);
+    box[1] = make_float4(-3.4e38f, -3.4e38f, -3.4e38f, 0.f);
+}
+
+// The run of configurations [t_lo, t_hi) that warp w of a group steps in traj_step, ascending with
+// w: the first warp, busy with the placement gradient, takes none, or a third where there are but
+// two; point to point has none and deals equal runs.
+template <bool kP2P, int kPpc>
 __device__ __forceinline__ void step_run(int C, int w, int& t_lo, int& t_hi) {
-    const int run = (C + kGrpWarps<kPpc> - 2) / (kGrpWarps<kPpc> - 1);
-    t_lo = w > 0 ? min(C, (w - 1) * run) : C;
-    t_hi = min(C, t_lo + run);
+    constexpr int kWarps = kGrpWarps<kPpc>;
+    const int first = kP2P ? (C + kWarps - 1) / kWarps : kWarps == 2 ? C / 3 : 0;
+    const int run = (C - first + kWarps - 2) / (kWarps - 1);
+    t_lo = w > 0 ? min(C, first + (w - 1) * run) : 0;
+    t_hi = w > 0 ? min(C, t_lo + run) : first;
 }
 
 // Evaluate the whole particle: kinematics of the grasp/place configurations and the placed
@@ -822,7 +835,7 @@ __device__ __forceinline__ void step_run(int C, int w, int& t_lo, int& t_hi) {
 // the placement gradient without its collision terms).
 template <bool kP2P, int kTile, int kPpc>
 __device__ void traj_evaluate(const TrajScalars& sc, const LaneSpheres& ls, const float4* cub, const float4* osph,
-                              float4* aabb, TShared& sh, TWarp* tws, SpecialFrames* sp, float* q, float* rows,
+                              const float4* aabb, TShared& sh, TWarp* tws, SpecialFrames* sp, float* q, float* rows,
                               float* disp, float* cblk, __half2* cgap, unsigned char* state, float* ctopm,
                               __half* ctop, bool grad, bool last) {
     constexpr int kWarps = kGrpWarps<kPpc>;
@@ -889,7 +902,7 @@ __device__ void traj_evaluate(const TrajScalars& sc, const LaneSpheres& ls, cons
                         }
                         for (int i = 0; i < 4; ++i) sh.pose[4 * lane + i] = sh.pose_prev[4 * lane + i] = pose[i];
                         block_cuboid(pose[0], pose[1], pose[2], pose[3], sc.half[lane], sh.blk[lane]);
-                        cuboid_aabb(sh.blk[lane], aabb + 64 * (t_words(sc.n_cub, sc.n_osph) - 1) + 2 * lane);
+                        cuboid_aabb(sh.blk[lane], sh.bbox[lane]);
                     } else if (lane < B) {   // point to point: the placed boxes stay empty
                         for (int i = 0; i < 4; ++i) sh.pose[4 * lane + i] = 0.f;
                     }
@@ -1044,7 +1057,7 @@ __device__ void traj_evaluate(const TrajScalars& sc, const LaneSpheres& ls, cons
     acc_max = warp_fmax(acc_max);
     if (lane == 0) tws[w].maxpen = acc_max;
     int t_lo, t_hi;
-    step_run<kPpc>(C, w, t_lo, t_hi);
+    step_run<kP2P, kPpc>(C, w, t_lo, t_hi);
     if (lane < 4 && t_lo < t_hi)   // for the step: the run's first row, then its last
         tws[w].edge[lane >> 1][lane & 1] = reinterpret_cast<const float4*>(q + 8 * (lane < 2 ? t_lo : t_hi - 1))[lane & 1];
     grp_sync<kPpc>();
@@ -1109,7 +1122,7 @@ __device__ __forceinline__ void traj_step(const TrajScalars& sc, TShared& sh, TW
     const int tid = grp_tid<kPpc>(), lane = tid & 31, w = tid >> 5;
     const int B = sc.B, C = sc.C, S = sc.S, n_pu = kP2P ? 0 : (8 * B + 31) / 32;
     int t_lo, t_hi;
-    step_run<kPpc>(C, w, t_lo, t_hi);
+    step_run<kP2P, kPpc>(C, w, t_lo, t_hi);
     const float tot_a = fx_value(sh.fx_tot[0]), tot_b = fx_value(sh.fx_tot[1]);
     const float s_arm = residual_scale(sh, 9 * B + 1, sc.sqw[4], tot_a);
     const float s_blk = residual_scale(sh, 9 * B + 2, sc.sqw[5], tot_b);
@@ -1135,7 +1148,7 @@ __device__ __forceinline__ void traj_step(const TrajScalars& sc, TShared& sh, TW
         const int t = t0 + lane;
         const bool in = t < t_hi;
         const float4* qv = reinterpret_cast<const float4*>(q + 8 * min(t, t_hi - 1));
-        const float4* pr = lane > 0 ? qv - 2 : t0 > t_lo ? tws[w].edge[2] : w > 1 ? tws[w - 1].edge[1] : qv;
+        const float4* pr = lane > 0 ? qv - 2 : t0 > t_lo ? tws[w].edge[2] : t0 > 0 ? tws[w - 1].edge[1] : qv;
         const float4* nx = t + 1 >= C ? qv : t + 1 < t_hi ? qv + 2 : tws[w + 1].edge[0];
         const float4 a0 = qv[0], a1 = qv[1], p0 = pr[0], p1 = pr[1], n0 = nx[0], n1 = nx[1];
         const float v[7] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z};
@@ -1277,23 +1290,16 @@ __device__ __forceinline__ void traj_path(const TrajScalars& sc, TShared& sh, co
     // no barrier: only thread 0 reads sh.path, sh.jl and sh.L afterwards
 }
 
-// Constants of a problem in its group's region that its particles share: the boxes of the
-// environment, the cuboids of the blocks at their initial poses, the kinematic rows.  The
-// environment tables are already there (smem_raw, laid out by the t_*_offset functions).  The
-// caller's next barrier orders the writes.
-template <int kPpc>
-__device__ __forceinline__ void traj_setup(const TrajScalars& sc, unsigned char* smem_raw) {
-    const float4* cub = reinterpret_cast<const float4*>(smem_raw + t_env_offset());
+// Boxes of a problem's environment by `threads` threads (tid of them); its tables are already in
+// shared memory.  The caller's next barrier orders the writes.
+__device__ __forceinline__ void env_setup(const TrajScalars& sc, unsigned char* env, int tid, int threads) {
+    const float4* cub = reinterpret_cast<const float4*>(env + t_env_offset());
     const float4* osph = cub + 4 * sc.n_cub;
-    float4* aabb = reinterpret_cast<float4*>(smem_raw + t_aabb_offset(sc.n_cub, sc.n_osph));
-    TShared& sh = *reinterpret_cast<TShared*>(smem_raw + t_shared_offset(sc.n_cub, sc.n_osph));
-    const int tid = grp_tid<kPpc>();
-    const float4 empty_lo = make_float4(3.4e38f, 3.4e38f, 3.4e38f, 0.f);   // an empty box: never a candidate
-    const float4 empty_hi = make_float4(-3.4e38f, -3.4e38f, -3.4e38f, 0.f);
+    float4* aabb = reinterpret_cast<float4*>(env + t_aabb_offset(sc.n_cub, sc.n_osph));
     const int n_cw = t_cub_words(sc.n_cub), n_w = t_words(sc.n_cub, sc.n_osph);
 #pragma unroll 1
-    for (int i = tid; i < 32 * n_w; i += kGrpThreads<kPpc>) {
-        const int o = i - 32 * n_cw, k = i - 32 * (n_w - 1) - kMaxB;   // environment sphere, block at its initial pose
+    for (int i = tid; i < 32 * (n_w - 1); i += threads) {
+        const int o = i - 32 * n_cw;   // environment sphere
         float4* box = &aabb[2 * i];
         if (i < sc.n_cub) {
             cuboid_aabb(&cub[4 * i], box);
@@ -1301,12 +1307,24 @@ __device__ __forceinline__ void traj_setup(const TrajScalars& sc, unsigned char*
             const float4 sp = osph[o];
             box[0] = make_float4(sp.x - sp.w, sp.y - sp.w, sp.z - sp.w, 0.f);
             box[1] = make_float4(sp.x + sp.w, sp.y + sp.w, sp.z + sp.w, 0.f);
-        } else if (k >= 0 && k < sc.B) {
-            block_cuboid(sc.init[k].x, sc.init[k].y, sc.init[k].z, sc.init[k].w, sc.half[k], sh.blk[kMaxB + k]);
-            cuboid_aabb(sh.blk[kMaxB + k], box);
         } else {
-            box[0] = empty_lo;
-            box[1] = empty_hi;
+            empty_box(box);
+        }
+    }
+}
+
+// Constants of a problem in its group's region that its particles share: the cuboids of the
+// blocks at their initial poses (the placed ones empty), the kinematic rows.
+template <int kPpc>
+__device__ __forceinline__ void group_setup(const TrajScalars& sc, TShared& sh) {
+    const int tid = grp_tid<kPpc>();
+    if (tid < 2 * kMaxB) {
+        const int k = tid - kMaxB;
+        if (k >= 0 && k < sc.B) {
+            block_cuboid(sc.init[k].x, sc.init[k].y, sc.init[k].z, sc.init[k].w, sc.half[k], sh.blk[tid]);
+            cuboid_aabb(sh.blk[tid], sh.bbox[tid]);
+        } else {
+            empty_box(sh.bbox[tid]);
         }
     }
     if (tid == 0) sh.inv_S = 1.f / (float)sc.S;
@@ -1321,19 +1339,20 @@ __device__ __forceinline__ void traj_setup(const TrajScalars& sc, unsigned char*
 
 // One particle of the trajectory stage by a group: load its state, run the descent (or the
 // single evaluation), write the outputs.  The problem's constants are already in shared memory
-// (traj_setup).  rows: the group's slot of the collision gradient rows.
+// (env_setup, group_setup).  rows: the group's slot of the collision gradient rows.
 template <bool kP2P, int kTile, int kPpc>
 __device__ __forceinline__ void traj_particle(const TrajScalars& sc, const LaneSpheres& ls, int p, int mode,
-                                              const TrajIO& io, float* rows, unsigned char* smem_raw) {
+                                              const TrajIO& io, float* rows, const unsigned char* env,
+                                              unsigned char* region) {
     constexpr int kThreads = kGrpThreads<kPpc>, kWarps = kGrpWarps<kPpc>;
-    const float4* cub = reinterpret_cast<const float4*>(smem_raw + t_env_offset());
+    const float4* cub = reinterpret_cast<const float4*>(env + t_env_offset());
     const float4* osph = cub + 4 * sc.n_cub;
-    float4* aabb = reinterpret_cast<float4*>(smem_raw + t_aabb_offset(sc.n_cub, sc.n_osph));
-    TShared& sh = *reinterpret_cast<TShared*>(smem_raw + t_shared_offset(sc.n_cub, sc.n_osph));
-    TWarp* tws = reinterpret_cast<TWarp*>(smem_raw + t_warp_offset(sc.n_cub, sc.n_osph));
-    float* q = reinterpret_cast<float*>(smem_raw + t_q_offset(sc.n_cub, sc.n_osph, kWarps));
-    SpecialFrames* sp = reinterpret_cast<SpecialFrames*>(smem_raw + t_sp_offset(sc.n_cub, sc.n_osph, sc.C, kWarps));
-    float* disp = reinterpret_cast<float*>(smem_raw + t_cache_offset(sc.n_cub, sc.n_osph, sc.C, sc.B, kWarps));
+    const float4* aabb = reinterpret_cast<const float4*>(env + t_aabb_offset(sc.n_cub, sc.n_osph));
+    TShared& sh = *reinterpret_cast<TShared*>(region);
+    TWarp* tws = reinterpret_cast<TWarp*>(region + t_warp_offset());
+    float* q = reinterpret_cast<float*>(region + t_q_offset(kWarps));
+    SpecialFrames* sp = reinterpret_cast<SpecialFrames*>(region + t_sp_offset(sc.C, kWarps));
+    float* disp = reinterpret_cast<float*>(region + t_cache_offset(sc.C, sc.B, kWarps));
     const int n_chunks = t_n_chunks(sc.C);
     float* cblk = disp + sc.C;
     __half2* cgap = reinterpret_cast<__half2*>(cblk + n_chunks);   // (static, moving) clearances
@@ -1468,21 +1487,24 @@ __device__ __forceinline__ bool stage_tables_grp(void* dst0, const void* src0, u
 // per group.  (kP2P: the point-to-point instantiation; kTile: the sphere tiling.)
 template <bool kP2P, int kTile, int kPpc>
 __global__ void __launch_bounds__(kTThreads, 2) k_traj(const __grid_constant__ Scalars sc, DevTables tab, int n, int mode,
-                                                       TrajIO io, int* err, int region) {
+                                                       TrajIO io, int* err, int region_bytes) {
     extern __shared__ __align__(16) unsigned char smem_all[];
     if (io.active && *io.active <= 0) return;   // stage 1 of this problem found no placement
-    unsigned char* smem_raw = smem_all + (size_t)grp_index<kPpc>() * region;
-    uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
-    float4* cub = reinterpret_cast<float4*>(smem_raw + t_env_offset());
+    // the environment, which the CTA's groups share, then their regions
+    unsigned char* region = smem_all + t_env_bytes(sc.n_cub, sc.n_osph) + (size_t)grp_index<kPpc>() * region_bytes;
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem_all);
+    float4* cub = reinterpret_cast<float4*>(smem_all + t_env_offset());
     float4* osph = cub + 4 * sc.n_cub;
-    TShared& sh = *reinterpret_cast<TShared*>(smem_raw + t_shared_offset(sc.n_cub, sc.n_osph));
+    TShared& sh = *reinterpret_cast<TShared*>(region);
     const int groups = gridDim.x * kPpc, slot = blockIdx.x * kPpc + grp_index<kPpc>();
-    if (stage_tables_grp<kPpc>(cub, tab.cub, (uint32_t)sc.n_cub * 64u, osph, tab.osph, (uint32_t)sc.n_osph * 16u, bar, err)) {
-        traj_setup<kPpc>(sc, smem_raw);
+    if (stage_tables(cub, tab.cub, (uint32_t)sc.n_cub * 64u, osph, tab.osph, (uint32_t)sc.n_osph * 16u, bar, err)) {
+        env_setup(sc, smem_all, threadIdx.x, kTThreads);
+        group_setup<kPpc>(sc, sh);
+        __syncthreads();
         const LaneSpheres ls = lane_spheres<kTile>(sc);
         float* rows = io.rows + (size_t)slot * sc.C * 16;
         for (int p = slot; p < n;) {
-            traj_particle<kP2P, kTile, kPpc>(sc, ls, p, mode, io, rows, smem_raw);
+            traj_particle<kP2P, kTile, kPpc>(sc, ls, p, mode, io, rows, smem_all, region);
             if (grp_tid<kPpc>() == 0) sh.particle = groups + atomicAdd(&io.work->next, 1);
             grp_sync<kPpc>();   // also: the outputs were read from the region before the next particle fills it
             p = sh.particle;
@@ -1509,16 +1531,17 @@ static_assert(sizeof(TrajScalars) % 16 == 0, "the batched kernel copies TrajScal
 // schedule.
 template <int kTile, int kPpc>
 __global__ void __launch_bounds__(kTThreads, 2) k_traj_batch(const TrajJob* __restrict__ jobs, int n_jobs, int n_items,
-                                                             int per_fetch, int mode, int* next, int region) {
+                                                             int per_fetch, int mode, int* next, int group_bytes) {
     extern __shared__ __align__(16) unsigned char smem_all[];
     __shared__ __align__(16) TrajScalars sc_arr[kPpc];
     __shared__ TrajIO io_arr[kPpc];
     __shared__ int s_item[kPpc], s_job[kPpc];
     const int g = grp_index<kPpc>(), tid = grp_tid<kPpc>();
-    unsigned char* smem_raw = smem_all + (size_t)g * region;
+    unsigned char* env = smem_all + (size_t)g * group_bytes;   // the group's environment, then its region
+    unsigned char* region = env;
     TrajScalars& sc_s = sc_arr[g];
     TrajIO& io_s = io_arr[g];
-    uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
+    uint64_t* bar = reinterpret_cast<uint64_t*>(env);
     int cur = -1;
     uint32_t uses = 0;
     for (;;) {
@@ -1547,12 +1570,14 @@ __global__ void __launch_bounds__(kTThreads, 2) k_traj_batch(const TrajJob* __re
             for (int i = tid; i < (int)(sizeof(TrajScalars) / 16); i += kGrpThreads<kPpc>) dst[i] = src[i];
             if (tid == 0) io_s = job.io;
             grp_sync<kPpc>();
-            float4* cub = reinterpret_cast<float4*>(smem_raw + t_env_offset());
+            float4* cub = reinterpret_cast<float4*>(env + t_env_offset());
             float4* osph = cub + 4 * sc_s.n_cub;
             if (!stage_tables_grp<kPpc>(cub, job.tab.cub, (uint32_t)sc_s.n_cub * 64u, osph, job.tab.osph,
                                   (uint32_t)sc_s.n_osph * 16u, bar, job.err, uses == 0, uses & 1u))
                 return;
-            traj_setup<kPpc>(sc_s, smem_raw);   // ordered by the first barrier of traj_particle
+            region = env + t_env_bytes(sc_s.n_cub, sc_s.n_osph);
+            env_setup(sc_s, env, tid, kGrpThreads<kPpc>);   // ordered by the first barrier of traj_particle
+            group_setup<kPpc>(sc_s, *reinterpret_cast<TShared*>(region));
             ++uses;
             cur = j;
         }
@@ -1562,19 +1587,14 @@ __global__ void __launch_bounds__(kTThreads, 2) k_traj_batch(const TrajJob* __re
         // a problem whose stage 1 found no placement has nothing to optimise
         const int p1 = (io_s.active && *io_s.active <= 0) ? p0 : min(p0 + per_fetch, job.n);
         for (int p = p0; p < p1; ++p) {
-            if (sc_s.kind == kKindP2P) traj_particle<true, kTile, kPpc>(sc_s, ls, p, mode, io_s, rows, smem_raw);
-            else traj_particle<false, kTile, kPpc>(sc_s, ls, p, mode, io_s, rows, smem_raw);
+            if (sc_s.kind == kKindP2P) traj_particle<true, kTile, kPpc>(sc_s, ls, p, mode, io_s, rows, env, region);
+            else traj_particle<false, kTile, kPpc>(sc_s, ls, p, mode, io_s, rows, env, region);
             grp_sync<kPpc>();
         }
     }
 }
 
 // ================================================================================== launchers
-// Shared memory of one group: the problem's layout, rounded to 128 bytes.
-static int t_region(size_t bytes) { return (int)((bytes + 127) & ~(size_t)127); }
-
-size_t traj_cta_smem_bytes(const TrajScalars& sc, int ppc) { return (size_t)t_region(traj_smem_bytes(sc, ppc)) * ppc; }
-
 // Two CTAs per SM share its shared memory; each has 1 KB of it reserved by the system.
 static cudaError_t sm_limits(int* sms, size_t* half_smem) {
     int dev = 0, smem = 0, reserved = 0;
@@ -1586,20 +1606,27 @@ static cudaError_t sm_limits(int* sms, size_t* half_smem) {
     return e;
 }
 
-// Particles per CTA where the caller leaves the choice: two, on 4 warps each, when the launch
-// has more particles than the SMs hold one to a CTA (2 CTAs per SM) and two CTAs with two
-// particles still fit an SM; otherwise one, on all 8 warps (fewer particles: each finishes
-// sooner; larger regions: two particles would leave an SM one CTA, 8 warps in place of 16).
-// Towers of more than kAutoBlocks blocks keep one too: their phases run through more of the
-// kernel's code at a time, and four particles in different phases miss the instruction cache
-// (4096 particles, 50 steps, one / two per CTA: 10 blocks 13.6 / 16.3 ms, 4 blocks 5.7 / 4.2 ms,
-// point to point 8.7 / 6.3 ms).
-constexpr int kAutoBlocks = 4;
-int traj_auto_ppc(size_t cta_bytes_2, long long particles, int blocks) {
+// Particles per CTA where the caller leaves the choice.  More than one when the launch has more
+// particles than the SMs then hold (2 CTAs per SM) and two such CTAs fit an SM; otherwise
+// fewer, on more warps each (fewer particles: each finishes sooner; larger regions: an SM would
+// hold one CTA, 8 warps in place of 16).
+// Towers of more than kAutoBlocks blocks keep one: their phases run through more of the kernel's
+// code at a time, and four particles in different phases miss the instruction cache.  4096
+// particles, 50 steps, one / two per CTA, ms: 2 blocks 4.1 / 2.7, 4 blocks 5.6 / 4.0, 6 blocks
+// 6.9 / 5.8, 8 blocks 9.2 / 9.0, 10 blocks 12.6 / 15.5.
+// Four take short trajectories (kShortC configurations; 1 block, 31 configurations, 700 / 4096
+// particles, two / four per CTA: 0.82 / 0.68 and 2.62 / 1.86 ms), and longer ones up to kMidC when
+// the launch has several rounds of them, as a particle on two warps runs long and the last ones
+// run alone (3 blocks, 187 configurations, 2048 / 4096 particles: 2.86 / 3.33 and 4.75 / 4.35 ms).
+// cta_bytes_2, cta_bytes_4: the shared memory of a CTA with 2 or 4 particles (0: not to be used).
+constexpr int kAutoBlocks = 6, kShortC = 48, kMidC = 192;
+int traj_auto_ppc(size_t cta_bytes_2, size_t cta_bytes_4, long long particles, int blocks, int C) {
     int sms = 0;
     size_t half = 0;
-    if (sm_limits(&sms, &half) != cudaSuccess) return 1;
-    return particles > 2LL * sms && cta_bytes_2 <= half && blocks <= kAutoBlocks ? 2 : 1;
+    if (sm_limits(&sms, &half) != cudaSuccess || blocks > kAutoBlocks) return 1;
+    const bool four = C <= kShortC ? particles > 4LL * sms : C <= kMidC && particles > 16LL * sms;
+    if (cta_bytes_4 && four && cta_bytes_4 <= std::min(half, kHalfSmem)) return 4;
+    return cta_bytes_2 && particles > 2LL * sms && cta_bytes_2 <= half ? 2 : 1;
 }
 
 template <int kTile, int kPpc>
@@ -1635,18 +1662,24 @@ int traj_batch_ctas_per_sm(size_t cta_bytes, int tiling, int ppc) {
 }
 
 int traj_ppc(const TrajScalars& sc, long long particles) {
-    return sc.particles_per_cta ? sc.particles_per_cta : traj_auto_ppc(traj_cta_smem_bytes(sc, 2), particles, sc.B);
+    if (sc.particles_per_cta) return sc.particles_per_cta;
+    // point to point keeps two (1024 / 4096 particles, two / four per CTA: 1.9 / 2.3 and 5.9 / 5.8 ms):
+    // its eight chunks, all near obstacles, are too few and too long for two warps
+    const bool four = !sc.sphere_tiling && sc.kind != kKindP2P;
+    return traj_auto_ppc(traj_cta_smem_bytes(sc, 2, false), four ? traj_cta_smem_bytes(sc, 4, false) : 0, particles, sc.B,
+                         sc.C);
 }
 
 template <bool kP2P>
 static int single_ctas(size_t dyn, int tiling, int ppc) {
+    if (ppc == 4) return occupancy(k_traj<kP2P, 0, 4>, dyn);
     if (ppc == 2) return tiling ? occupancy(k_traj<kP2P, 1, 2>, dyn) : occupancy(k_traj<kP2P, 0, 2>, dyn);
     return tiling ? occupancy(k_traj<kP2P, 1, 1>, dyn) : occupancy(k_traj<kP2P, 0, 1>, dyn);
 }
 
 int traj_ctas_per_sm(const TrajScalars& sc) {
     const int ppc = traj_ppc(sc, sc.Q);
-    const size_t dyn = traj_cta_smem_bytes(sc, ppc);
+    const size_t dyn = traj_cta_smem_bytes(sc, ppc, false);
     return sc.kind == kKindP2P ? single_ctas<true>(dyn, sc.sphere_tiling, ppc)
                                : single_ctas<false>(dyn, sc.sphere_tiling, ppc);
 }
@@ -1654,22 +1687,24 @@ int traj_ctas_per_sm(const TrajScalars& sc) {
 template <bool kP2P, int kTile, int kPpc>
 static cudaError_t traj_kernel(const Scalars& sc, DevTables t, int n, int mode, const TrajIO& io, int* err,
                                cudaStream_t st) {
-    const size_t dyn = traj_cta_smem_bytes(sc, kPpc);
+    const size_t dyn = traj_cta_smem_bytes(sc, kPpc, false);
     int sms = 0;
     size_t half = 0;
     cudaError_t e = sm_limits(&sms, &half);
     if (e == cudaSuccess) e = allow_max_dynamic_smem(k_traj<kP2P, kTile, kPpc>, dyn);
     if (e != cudaSuccess) return e;
-    const int resident = std::min(sms * (dyn <= half ? 2 : 1), kTrajSlots / kPpc);
+    const int resident = std::min(sms * (dyn <= half ? 2 : 1), traj_slots(sc.B, sc.C, sc.n_cub, sc.n_osph) / kPpc);
     const int grid = std::min((n + kPpc - 1) / kPpc, resident);
-    k_traj<kP2P, kTile, kPpc><<<grid, kTThreads, dyn, st>>>(sc, t, n, mode, io, err, (int)(dyn / kPpc));
+    k_traj<kP2P, kTile, kPpc><<<grid, kTThreads, dyn, st>>>(sc, t, n, mode, io, err, (int)t_region(sc.C, sc.B, kPpc));
     return cudaGetLastError();
 }
 
 template <bool kP2P>
 static cudaError_t traj_dispatch(const Scalars& sc, DevTables t, int n, int mode, const TrajIO& io, int* err,
                                  cudaStream_t st) {
-    if (traj_ppc(sc, n) == 2)
+    const int ppc = traj_ppc(sc, n);
+    if (ppc == 4) return traj_kernel<kP2P, 0, 4>(sc, t, n, mode, io, err, st);
+    if (ppc == 2)
         return sc.sphere_tiling ? traj_kernel<kP2P, 1, 2>(sc, t, n, mode, io, err, st)
                                 : traj_kernel<kP2P, 0, 2>(sc, t, n, mode, io, err, st);
     return sc.sphere_tiling ? traj_kernel<kP2P, 1, 1>(sc, t, n, mode, io, err, st)

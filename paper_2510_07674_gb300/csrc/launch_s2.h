@@ -28,13 +28,15 @@ struct TrajIO {
     int init_multipliers;   // descent starts from lambda = 0, mu = mu0
     const int* active;  // optional device word: when it holds 0 or less the launch does nothing (the
                         // trajectory stage of a problem whose stage 1 found no placement)
-    float* rows;        // [kTrajSlots][C][16] scratch (required): the collision gradient rows of the
+    float* rows;        // [traj_slots][C][16] scratch (required): the collision gradient rows of the
                         // particle each resident group works on
     TrajWork* work;   // the launch's work counters (required by launch_traj), zero between launches
 };
-// Particle groups resident at once: two CTAs of two groups on each of 152 SMs; a launch on a
-// part with more SMs keeps to this many.
+// Particle groups resident at once: two CTAs of two groups on each of 152 SMs, or of four where
+// the problem is small enough (traj_slots); a launch on a part with more SMs keeps to as many.
 constexpr int kTrajSlots = 608;
+constexpr size_t kHalfSmem = 228 * 512 - 1024;   // shared memory of each of two CTAs on an SM
+int traj_slots(int B, int C, int n_cub, int n_osph);
 enum TrajModeHost { kTrajModeEval = 0, kTrajModeDescend = 1, kTrajModeCheck = 2 };
 
 // One problem of a batched trajectory launch (device array, sorted by `first`).
@@ -48,9 +50,10 @@ struct TrajJob {
 };
 
 // Particles per CTA of a launch of that many particles: the problem's setting, or the
-// launcher's choice (traj_auto_ppc, given the shared memory of a CTA with two particles and the blocks).
+// launcher's choice (traj_auto_ppc, given the shared memory of a CTA with two and with four
+// particles, 0 where that shape is not to be used, the blocks and the configurations).
 int traj_ppc(const TrajScalars& sc, long long particles);
-int traj_auto_ppc(size_t cta_bytes_2, long long particles, int blocks);
+int traj_auto_ppc(size_t cta_bytes_2, size_t cta_bytes_4, long long particles, int blocks, int C);
 // IK at grasp/place poses + interpolation; particle p lifts placement p % n_place.  With
 // ctl != nullptr the attempt counter, the placement count and the Philox key are read on the
 // device (ctl->t_attempt, ctl->n_place, ctl->seed) in place of `attempt`, `n_place` and
@@ -73,6 +76,7 @@ int traj_batch_ctas_per_sm(size_t cta_bytes, int tiling, int ppc);
 // shape (0 if it does not fit).
 int traj_ctas_per_sm(const TrajScalars& sc);
 // Dynamic shared memory of one trajectory CTA with ppc particles.
-size_t traj_cta_smem_bytes(const TrajScalars& sc, int ppc);
+// (batched: each group has its own environment tables; otherwise the CTA's groups share them).
+size_t traj_cta_smem_bytes(const TrajScalars& sc, int ppc, bool batched);
 
 }  // namespace spasm

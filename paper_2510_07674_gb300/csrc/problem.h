@@ -49,7 +49,7 @@ struct spasm_problem {
     int *d_tsat = nullptr, *d_tnsat = nullptr, *d_tbest = nullptr;
     float *d_rq = nullptr, *d_rcost = nullptr;   // returned solutions
     int* d_rsucc = nullptr;
-    float* d_rows = nullptr;             // the trajectory kernel's gradient rows (kTrajSlots x C x 16)
+    float* d_rows = nullptr;             // the trajectory kernel's gradient rows (traj_slots x C x 16)
     spasm::TrajWork* d_work = nullptr;   // and work counters
     unsigned long long* d_tests = nullptr;   // [tests run, configurations culled] by the trajectory kernel
     bool optimized = false;
