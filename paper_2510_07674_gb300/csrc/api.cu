@@ -79,7 +79,7 @@ static void free_all(spasm_problem* pr) {
                     pr->d_idx, pr->d_sat, pr->d_nsat, pr->d_best, pr->d_place, pr->d_q, pr->d_lam,
                     pr->d_mu, pr->d_metrics, pr->d_tmasked, pr->d_tsat, pr->d_tnsat, pr->d_tbest, pr->d_rq,
                     pr->d_rcost, pr->d_rsucc, pr->d_cub64, pr->d_osph64, pr->d_rmet64, pr->d_tests, pr->d_sc, pr->d_chkacc,
-                    pr->d_ctl, pr->d_rows, pr->d_work};
+                    pr->d_ctl, pr->d_rows, pr->d_work, pr->d_chkval};
     for (void* p : ptrs)
         if (p) cudaFreeAsync(p, pr->stream);
     for (cudaEvent_t e : pr->ev)
@@ -139,6 +139,7 @@ static void for_each_buffer(spasm_problem* pr, int B, int C, int n_cub, int n_os
     f(pr->d_ctl, 1);
     f(pr->d_rows, (size_t)traj_slots(B, C, n_cub, n_osph) * C * 16);
     f(pr->d_work, 1);
+    f(pr->d_chkval, P * (size_t)C);
 }
 
 extern "C" spasm_status spasm_problem_bytes(const spasm_obstacles* obs, const spasm_goal* goal, const spasm_params* prm,
@@ -361,6 +362,20 @@ static spasm_status create_problem_impl(const spasm_robot* robot, const spasm_ob
             zz += 2.0 * hh[2];
         }
         q.grasp_off = goal->grasp_off; q.eps = prm->eps; q.eps_start = prm->eps_start;
+        // the FP32 screen's margin: 2e-5 (335 rounding steps) of the scene's extent, the arm's length with
+        // its largest sphere or held block and the farthest obstacle point from the origin
+        auto norm3 = [](const double* v) { return std::sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]); };
+        double arm = 0.0, far = 0.0, held = 0.0;
+        for (int k = 0; k < 7; ++k) arm += std::fabs(q.a[k]) + std::fabs(q.d[k]);
+        double tip = 0.0;
+        for (int i = 0; i < sc.n_rsph; ++i) tip = std::fmax(tip, norm3(q.rsph[i]) + std::fabs(q.rsph[i][3]));
+        for (int i = 0; i < B; ++i) {
+            held = std::fmax(held, 2.0 * norm3(q.half[i]) + std::fabs(q.grasp_off));
+            far = std::fmax(far, norm3(q.init[i]) + norm3(q.half[i]));
+        }
+        for (int o = 0; o < sc.n_cub; ++o) far = std::fmax(far, norm3(obs->cuboid + 15 * o) + norm3(obs->cuboid + 15 * o + 12));
+        for (int o = 0; o < sc.n_osph; ++o) far = std::fmax(far, norm3(obs->sphere + 4 * o) + std::fabs(obs->sphere[4 * o + 3]));
+        q.margin = (float)(2e-5 * (arm + norm3(q.ee_p) + tip + held + far));
     }
     pr->host_osph.assign(obs->sphere, obs->sphere + 4 * (size_t)sc.n_osph);
 
@@ -645,8 +660,8 @@ extern "C" spasm_status spasm_traj_check(spasm_problem_t pr, int n, const float*
     const int P = pr->sc.P, C = pr->sc.C;
     for (int off = 0; off < n; off += P) {
         const int k = n - off < P ? n - off : P;
-        SPASM_CUDA(launch_check64(pr->s64, pr->d_cub64, pr->d_osph64, q + (size_t)off * C * 8, nullptr, k,
-                                  metrics + (size_t)off * 6, ok + off, pr->d_chkacc, pr->stream));
+        SPASM_CUDA(launch_check64(pr->s64, pr->sc, pr->tab, pr->d_cub64, pr->d_osph64, q + (size_t)off * C * 8, nullptr, k,
+                                  metrics + (size_t)off * 6, ok + off, pr->d_chkval, pr->d_chkacc, pr->stream));
     }
     return SPASM_OK;
 }

@@ -2,7 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
-#include "common.cuh"
+#include "launch.h"
 
 namespace spasm {
 
@@ -16,13 +16,16 @@ struct Scalars64 {
     double half[kMaxB][3], hmin[kMaxB], init[kMaxB][4], zt[kMaxB];
     double grasp_off, eps, eps_start;
     int p2p;   // point to point: one segment, no placement
+    float margin;   // bound on the error of a sphere-obstacle distance evaluated in FP32
 };
 
-// Per-solution accumulator of the split check (zeroed once at allocation; the check leaves it
-// zeroed).
+// Per-solution accumulator of the check (zeroed once at allocation; the check leaves its
+// counters and maxima zeroed).
 struct CheckAcc {
     unsigned long long mp;   // largest arm / held-block penetration (bit pattern of a non-negative double)
     double pp, ms, mt, mD, mz;
+    double pose[kMaxB][5];   // placed blocks: x, y, z, cos yaw, sin yaw
+    unsigned top;            // largest FP32 value of the screen (an ordered key, 0 below every float)
     int viol;                // a joint outside its limits
     int count;               // slices done
 };
@@ -30,9 +33,11 @@ struct CheckAcc {
 // cub: n_cub x 4 x double4 (centre, then R columns with half extents); osph: n_osph x double4.
 // q: P x C x 8 floats; n_sol: device count of the rows that hold solutions (rows from
 // min(*n_sol, P) on get ok = 0 and keep their metrics), or nullptr when all P rows do.
+// sc, tab: the FP32 constants and tables; val: P x C floats of scratch.
 // metrics: P x 6 (max arm/held penetration, max grasp error, max tilt, placement max
 // penetration, max CoM distance, max height error); ok: P flags.
-cudaError_t launch_check64(const Scalars64& s, const void* cub, const void* osph, const float* q, const int* n_sol, int P,
-                           double* metrics, int* ok, CheckAcc* acc, cudaStream_t st);
+cudaError_t launch_check64(const Scalars64& s, const Scalars& sc, DevTables tab, const void* cub, const void* osph,
+                           const float* q, const int* n_sol, int P, double* metrics, int* ok, float* val, CheckAcc* acc,
+                           cudaStream_t st);
 
 }  // namespace spasm

@@ -215,8 +215,8 @@ spasm_status traj_select_loop(spasm_problem* pr, cudaStream_t s, cudaGraphCondit
     SPASM_CUDA(cudaGetLastError());
     return SPASM_OK;
 }
-// begin + finish (3) once; lift (2), descent, select and loop control per attempt
-constexpr int kTrajFixedKernels = 4;
+// begin + finish (4) once; lift (2), descent, select and loop control per attempt
+constexpr int kTrajFixedKernels = 5;
 constexpr int kTrajAttemptKernels = 5;
 
 // Captures what `enqueue` puts on `cap` into a graph and instantiates it.
@@ -339,8 +339,8 @@ spasm_status spasm::enqueue_finish(spasm_problem* pr, cudaStream_t s) {
                                              pr->d_rcost, pr->d_rsucc);
     SPASM_CUDA(cudaGetLastError());
     // FP64 re-evaluation of the returned solutions decides their success flags
-    SPASM_CUDA(launch_check64(pr->s64, pr->d_cub64, pr->d_osph64, pr->d_rq, pr->d_tnsat, sc.P, pr->d_rmet64,
-                              pr->d_rsucc, pr->d_chkacc, s));
+    SPASM_CUDA(launch_check64(pr->s64, sc, pr->tab, pr->d_cub64, pr->d_osph64, pr->d_rq, pr->d_tnsat, sc.P, pr->d_rmet64,
+                              pr->d_rsucc, pr->d_chkval, pr->d_chkacc, s));
     return SPASM_OK;
 }
 

@@ -72,7 +72,8 @@ struct spasm_problem {
     double* d_cub64 = nullptr;
     double* d_osph64 = nullptr;
     double* d_rmet64 = nullptr;
-    spasm::CheckAcc* d_chkacc = nullptr;   // accumulators of the split FP64 check (P)
+    spasm::CheckAcc* d_chkacc = nullptr;   // accumulators of the FP64 check (P)
+    float* d_chkval = nullptr;             // its screen's values (P x C)
     // statistics and timing
     spasm_stats stats{};
     bool timing = false;
