@@ -127,21 +127,9 @@ struct JobList {
     size_t cta_bytes = 0;   // shared memory of a CTA with ppc particles of the largest problem
 };
 
-// ppc 0: the launcher's choice over all particles.
 JobList make_jobs(spasm_problem_t* prs, const std::vector<int>& live, int per_fetch, int mode, int k_steps,
                   bool init_multipliers, int ppc) {
     JobList L;
-    if (ppc == 0) {
-        size_t two = 0;
-        long long particles = 0;
-        int blocks = 0;
-        for (int i : live) {
-            blocks = std::max(blocks, prs[i]->sc.B);
-            two = std::max(two, traj_cta_smem_bytes(prs[i]->sc, 2, true) + kBatchStaticSmem);
-            particles += prs[i]->sc.Q;
-        }
-        ppc = traj_auto_ppc(two, 0, particles, blocks, 0);
-    }
     L.ppc = ppc;
     for (int i : live) {
         spasm_problem* pr = prs[i];
@@ -248,6 +236,52 @@ spasm_status spasm::enqueue_batch(const BatchLaunch& bl, cudaStream_t s) {
     return SPASM_OK;
 }
 
+spasm::BatchSet::~BatchSet() {
+    if (fork) cudaEventDestroy(fork);
+    if (join) cudaEventDestroy(join);
+    if (side) cudaStreamDestroy(side);
+}
+
+spasm_status spasm::prepare_batches(spasm_problem_t* prs, const std::vector<int>& order, const spasm_batch_config& cfg,
+                                    cudaStream_t s, BatchSet& set) {
+    if (cfg.particles_per_cta) return prepare_batch(prs, order, cfg, s, set.launch[0]);
+    std::vector<int> by[2];   // one and two particles per CTA
+    long long particles = 0;
+    for (int i : order) particles += prs[i]->sc.Q;
+    for (int i : order) {
+        const Scalars& sc = prs[i]->sc;
+        const size_t two = traj_cta_smem_bytes(sc, 2, true) + kBatchStaticSmem;
+        by[traj_auto_ppc(two, 0, particles, sc.B, sc.C) - 1].push_back(i);
+    }
+    int n = 0;
+    for (int k = 0; k < 2; ++k) {
+        if (by[k].empty()) continue;
+        spasm_batch_config c = cfg;
+        c.particles_per_cta = k + 1;
+        SPASM_TRY(prepare_batch(prs, by[k], c, s, set.launch[n++]));
+    }
+    if (n == 2) {
+        SPASM_CUDA(cudaStreamCreateWithFlags(&set.side, cudaStreamNonBlocking));
+        SPASM_CUDA(cudaEventCreateWithFlags(&set.fork, cudaEventDisableTiming));
+        SPASM_CUDA(cudaEventCreateWithFlags(&set.join, cudaEventDisableTiming));
+    }
+    return SPASM_OK;
+}
+
+spasm_status spasm::enqueue_batches(const BatchSet& set, cudaStream_t s) {
+    if (set.side) {
+        SPASM_CUDA(cudaEventRecord(set.fork, s));
+        SPASM_CUDA(cudaStreamWaitEvent(set.side, set.fork, 0));
+    }
+    SPASM_TRY(enqueue_batch(set.launch[0], s));
+    if (set.side) {
+        SPASM_TRY(enqueue_batch(set.launch[1], set.side));
+        SPASM_CUDA(cudaEventRecord(set.join, set.side));
+        SPASM_CUDA(cudaStreamWaitEvent(s, set.join, 0));
+    }
+    return SPASM_OK;
+}
+
 extern "C" spasm_status spasm_batch_default_config(spasm_batch_config* cfg) {
     if (!cfg) return fail(SPASM_ERR_INVALID, "null config");
     cfg->per_fetch = 1;
@@ -268,7 +302,7 @@ extern "C" spasm_status spasm_optimize_batch(spasm_problem_t* prs, int n, void* 
         cfg = *cfg_in;
         SPASM_TRY(check_config(cfg));
     } else {
-        cfg.particles_per_cta = 0;   // chosen by prepare_batch
+        cfg.particles_per_cta = 0;   // chosen by prepare_batches
     }
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     std::vector<int> todo, all(n);
@@ -279,8 +313,8 @@ extern "C" spasm_status spasm_optimize_batch(spasm_problem_t* prs, int n, void* 
         all[i] = i;
     }
     const std::vector<int> order = job_order(prs, all, cfg.order);
-    BatchLaunch bl;
-    SPASM_TRY(prepare_batch(prs, order, cfg, s, bl));
+    BatchSet bl;
+    SPASM_TRY(prepare_batches(prs, order, cfg, s, bl));
     // one graph: stage 1 of the problems not yet placed, the first lift of every problem, one
     // persistent trajectory launch over all particles, then each problem's selection, re-lift
     // loop and FP64 check; problems whose stage 1 kept nothing skip stage 2 on the device
@@ -291,7 +325,7 @@ extern "C" spasm_status spasm_optimize_batch(spasm_problem_t* prs, int n, void* 
         SPASM_TRY(br.fork());
         for (int i = 0; i < n; ++i) SPASM_TRY(enqueue_traj_lift(prs[i], br[i]));
         SPASM_TRY(br.join());
-        SPASM_TRY(enqueue_batch(bl, c));
+        SPASM_TRY(enqueue_batches(bl, c));
         SPASM_TRY(br.fork());
         for (int i = 0; i < n; ++i) {
             SPASM_TRY(enqueue_traj_retry(prs[i], br[i]));

@@ -146,10 +146,25 @@ struct BatchLaunch {
     ~BatchLaunch();
 };
 // Builds and uploads (on s, asynchronously) the work list of problems prs[order[k]], each with
-// its own K_traj steps and its placement count as the gate.  cfg.particles_per_cta 0 leaves
-// that choice to the launcher (traj_auto_ppc over all particles).
+// its own K_traj steps and its placement count as the gate.
 spasm_status prepare_batch(spasm_problem_t* prs, const std::vector<int>& order, const spasm_batch_config& cfg,
                            cudaStream_t s, BatchLaunch& bl);
+// The launches of a batch whose particles per CTA are left to the library: the problems that run
+// best with one particle per CTA in one, those with two in another, which fills the SMs as the
+// first drains (the same bits either way).
+struct BatchSet {
+    BatchLaunch launch[2];   // the second empty where one shape takes all
+    cudaStream_t side = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+    BatchSet() = default;
+    BatchSet(const BatchSet&) = delete;
+    BatchSet& operator=(const BatchSet&) = delete;
+    ~BatchSet();
+};
+// cfg.particles_per_cta 0: as above; 1 or 2: one launch of that shape.
+spasm_status prepare_batches(spasm_problem_t* prs, const std::vector<int>& order, const spasm_batch_config& cfg,
+                             cudaStream_t s, BatchSet& set);
+spasm_status enqueue_batches(const BatchSet& set, cudaStream_t s);
 // Enqueues the launch (resetting its work counter first).
 spasm_status enqueue_batch(const BatchLaunch& bl, cudaStream_t s);
 // Reads what the device loops left (attempts, counts, counters, success flags, the error

@@ -164,9 +164,9 @@ void scheduler_loop(spasm_server* sv) {
         int status = SPASM_OK;
         std::string msg;
         {
-            BatchLaunch bl;
-            status = prepare_batch(prs.data(), order, cfg, st, bl);
-            if (status == SPASM_OK) status = enqueue_batch(bl, st);
+            BatchSet bl;
+            status = prepare_batches(prs.data(), order, cfg, st, bl);
+            if (status == SPASM_OK) status = enqueue_batches(bl, st);
             for (auto& r : active)
                 if (status == SPASM_OK) status = enqueue_traj_epoch_end(r->pr, st);
             if (status == SPASM_OK && cudaStreamSynchronize(st) != cudaSuccess) status = SPASM_ERR_CUDA;
