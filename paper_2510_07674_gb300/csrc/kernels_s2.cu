@@ -223,6 +223,7 @@ __device__ __forceinline__ LaneSpheres lane_spheres(const Scalars& sc) {
 // the lane also returns a world box (lo xyz, hi xyz) that holds every sphere of link k (and of
 // the held block, at k = 7 with `want_h`): the link-frame box of those spheres carried by the
 // frame, i.e. centre R c + o and half extents |R| h.
+template <bool kP2P>
 __device__ __forceinline__ void chunk_fk(const TrajScalars& sc, const TShared& sh, const float* __restrict__ q, int t_c, int b,
                                          bool write, bool want_h, float4 (*F_c)[3], float2 (*Z_c)[3], float4* H_c,
                                          float* box) {
@@ -241,7 +242,7 @@ __device__ __forceinline__ void chunk_fk(const TrajScalars& sc, const TShared& s
         A[6] = sa * st; A[7] = sa * ct; A[8] = ca;
         bv[0] = row.z; bv[1] = -sa * row.w; bv[2] = ca * row.w;
     }
-#pragma unroll 1
+#pragma unroll(kP2P ? 3 : 1)
     for (int off = 1; off < 8; off <<= 1) {
         float L[9], lb[3];
 #pragma unroll
@@ -374,7 +375,7 @@ __device__ __forceinline__ float warp_sums(float v[N]) {
 // The environment and the blocks share one cull loop and one test loop, and the kernel keeps
 // its other loops rolled: with four particles per SM in different phases the instruction cache
 // is what the warps compete for.
-template <int kTile>
+template <bool kP2P, int kTile>
 __device__ __forceinline__ int chunk_collisions(const TrajScalars& sc, const LaneSpheres& ls,
                                                  const float4* __restrict__ cub, const float4* __restrict__ osph,
                                                  const float4* aabb, TShared& sh, TWarp& tw, float* rows, int t0,
@@ -413,12 +414,13 @@ __device__ __forceinline__ int chunk_collisions(const TrajScalars& sc, const Lan
     // the blocks below it by at most the largest motion among them
     const int top = b_last - 1;
     const int n_cw = t_cub_words(sc.n_cub), n_w = t_words(sc.n_cub, sc.n_osph);
-    const int wd0 = skip & kStateSkipStatic ? n_w - 1 : 0;
+    // the words to look at; point to point has no blocks
+    const int wd0 = skip & kStateSkipStatic ? n_w - 1 : 0, wd1 = kP2P ? n_w - 1 : n_w;
     float clear = 3.4e38f, clear_m = 3.4e38f;
     uint32_t any = 0u;
 #pragma unroll 1
-    for (int wd = wd0; wd < n_w; ++wd) {
-        const bool blocks = wd == n_w - 1;
+    for (int wd = wd0; wd < wd1; ++wd) {
+        const bool blocks = !kP2P && wd == n_w - 1;
         const float4* box = blocks ? sh.bbox[0] : aabb + 64 * wd;
         const float4 clo = box[2 * lane], chi = box[2 * lane + 1];
         const float s1 = fmaxf(fmaxf(fmaxf(clo.x - hi_x, lo_x - chi.x), fmaxf(clo.y - hi_y, lo_y - chi.y)),
@@ -460,17 +462,17 @@ __device__ __forceinline__ int chunk_collisions(const TrajScalars& sc, const Lan
     }
     const unsigned has = __ballot_sync(0xffffffffu, any != 0u);   // bit 8c: configuration c has a candidate
     clearance = warp_fmin(clear);
-    clearance_moving = warp_fmin(clear_m);
+    clearance_moving = kP2P ? 3.4e38f : warp_fmin(clear_m);
     {
         // the top block: the gap from each link box of the configurations it concerns
         float ct = 3.4e38f;
-        if (top >= 0 && top < b_lane) {
+        if (!kP2P && top >= 0 && top < b_lane) {
             const float4 blo = sh.bbox[top][0], bhi = sh.bbox[top][1];
             const float g = fmaxf(fmaxf(fmaxf(blo.x - lb[3], lb[0] - bhi.x), fmaxf(blo.y - lb[4], lb[1] - bhi.y)),
                                   fmaxf(blo.z - lb[5], lb[2] - bhi.z));
             if (g > 0.f) ct = g;   // an overlapping box is tested against the spheres, which give the gap
         }
-        clearance_top = warp_fmin(ct);
+        clearance_top = kP2P ? 3.4e38f : warp_fmin(ct);
     }
     __syncwarp();
 
@@ -505,8 +507,8 @@ __device__ __forceinline__ int chunk_collisions(const TrajScalars& sc, const Lan
         visits = 0;
 
 #pragma unroll 1
-        for (int wd = wd0; wd < n_w; ++wd) {
-            const bool blocks = wd == n_w - 1;
+        for (int wd = wd0; wd < wd1; ++wd) {
+            const bool blocks = !kP2P && wd == n_w - 1;
             unsigned m = tw.mask[ci][wd];
             visits += __popc(m);
 #pragma unroll 1
@@ -588,32 +590,44 @@ __device__ __forceinline__ int chunk_collisions(const TrajScalars& sc, const Lan
         hits |= 1u << ci;
         if (!grad) continue;
 
-        // backward: dC/dq_k = sum_s z_k . ((c_s - o_k) x g_s) over spheres on links >= k, two joints
-        // (arm- and block-group torques of each) per round of a rolled loop: the seventh joint's
-        // partner k = 7 has no axis and stays zero
-#pragma unroll 1
-        for (int k0 = 0; k0 < 8; k0 += 2) {
-            float v[4] = {0.f, 0.f, 0.f, 0.f};   // arm k0, arm k0 + 1, block k0, block k0 + 1
+        // backward: dC/dq_k = sum_s z_k . ((c_s - o_k) x g_s) over spheres on links >= k
+        auto torque = [&](int k, float& arm, float& blk) {
+            const float4* f = tw.F[ci][k + 1];
+            const float4 f0 = f[0], f1 = f[1], f2 = f[2];
+            const float ox = f0.w, oy = f1.w, oz = f2.w;
+            const float zx = f0.z, zy = f1.z, zz = f2.z;
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int k = k0 + i;
-                if (i == 1 && k0 == 6) continue;
-                const float4* f = tw.F[ci][k + 1];
-                const float4 f0 = f[0], f1 = f[1], f2 = f[2];
-                const float ox = f0.w, oy = f1.w, oz = f2.w;
-                const float zx = f0.z, zy = f1.z, zz = f2.z;
-#pragma unroll
-                for (int sl = 0; sl < kSlots; ++sl) {
-                    const int lk = isblk[sl] ? 7 : ls.link[sl];
-                    if (!any_hit || !act[sl] || lk < k + 1) continue;
-                    const float vx = cx[sl] - ox, vy = cy[sl] - oy, vz = cz[sl] - oz;
-                    const float mm = zx * (vy * gz[sl] - vz * gy[sl]) + zy * (vz * gx[sl] - vx * gz[sl]) +
-                                     zz * (vx * gy[sl] - vy * gx[sl]);
-                    if (isblk[sl]) v[2 + i] += mm; else v[i] += mm;
-                }
+            for (int sl = 0; sl < kSlots; ++sl) {
+                const int lk = isblk[sl] ? 7 : ls.link[sl];
+                if (!any_hit || !act[sl] || lk < k + 1) continue;
+                const float vx = cx[sl] - ox, vy = cy[sl] - oy, vz = cz[sl] - oz;
+                const float mm = zx * (vy * gz[sl] - vz * gy[sl]) + zy * (vz * gx[sl] - vx * gz[sl]) +
+                                 zz * (vx * gy[sl] - vy * gx[sl]);
+                if (isblk[sl]) blk += mm; else arm += mm;
             }
-            const float torque = warp_sums<4>(v);   // lane 8 i: value i
-            if ((lane & 7) == 0) rows[16 * t + (lane >> 4) * 8 + k0 + ((lane >> 3) & 1)] = torque;
+        };
+        if (kP2P) {
+            // most configurations penetrate something and the rest of the code is small: all joints at
+            // once, one chain of exchanges
+            float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, none = 0.f;
+#pragma unroll
+            for (int k = 0; k < 7; ++k) torque(k, v[k], none);
+            const float sum = warp_sums<8>(v);   // lane 4 i: value i
+            if ((lane & 3) == 0) {
+                rows[16 * t + (lane >> 2)] = sum;
+                rows[16 * t + 8 + (lane >> 2)] = 0.f;
+            }
+        } else {
+            // two joints (arm- and block-group torques of each) per round of a rolled loop: the seventh
+            // joint's partner k = 7 has no axis and stays zero
+#pragma unroll 1
+            for (int k = 0; k < 8; k += 2) {
+                float v[4] = {0.f, 0.f, 0.f, 0.f};   // arm k, arm k + 1, block k, block k + 1
+                torque(k, v[0], v[2]);
+                if (k < 6) torque(k + 1, v[1], v[3]);
+                const float sum = warp_sums<4>(v);   // lane 8 i: value i
+                if ((lane & 7) == 0) rows[16 * t + (lane >> 4) * 8 + k + ((lane >> 3) & 1)] = sum;
+            }
         }
     }
     if (lane == 0) {
@@ -625,6 +639,7 @@ __device__ __forceinline__ int chunk_collisions(const TrajScalars& sc, const Lan
     // the tests' gaps join the clearances of a half without a penetration
     if (hits && lane == 0) atomicOr(&sh.hit[(t0 - 1) >> 5], hits << ((t0 - 1) & 31));
     clearance = fminf(clearance, warp_fmin(gap_s));
+    if (kP2P) return hits ? kStateZeroMoving : kStateZero;
     clearance_moving = fminf(clearance_moving, warp_fmin(gap_m));
     clearance_top = fminf(clearance_top, warp_fmin(gap_t));
     return (__any_sync(0xffffffffu, hit_s) ? 0 : kStateZeroStatic) | (__any_sync(0xffffffffu, hit_m) ? 0 : kStateZeroMoving);
@@ -1015,7 +1030,7 @@ __device__ void traj_evaluate(const TrajScalars& sc, const LaneSpheres& ls, cons
             b_c = seg >> 1;
         }
         float box[6];
-        chunk_fk(sc, sh, q, t_c, b_c, write, want_h, tws[w].F[c], special ? sp[si].Z : nullptr,
+        chunk_fk<kP2P>(sc, sh, q, t_c, b_c, write, want_h, tws[w].F[c], special ? sp[si].Z : nullptr,
                  special ? sp[si].H : tws[w].H[c], box);
         if (special) continue;
         __syncwarp();
@@ -1023,7 +1038,7 @@ __device__ void traj_evaluate(const TrajScalars& sc, const LaneSpheres& ls, cons
         float clearance, clearance_moving, clearance_top, c2[2] = {0.f, 0.f};
         int n_cand;
         const int skip = state[chk];
-        const int zero = chunk_collisions<kTile>(sc, ls, cub, osph, aabb, sh, tws[w], rows, t0, nc, seg_c, skip, grad, box,
+        const int zero = chunk_collisions<kP2P, kTile>(sc, ls, cub, osph, aabb, sh, tws[w], rows, t0, nc, seg_c, skip, grad, box,
                                                  c2[0], c2[1], acc_max, n_cand, clearance, clearance_moving,
                                                  clearance_top);
         if (zero != kStateZero) {
