@@ -3,9 +3,16 @@
 // One CTA of 1024 threads:  (1) costs become order-preserving 32-bit keys in shared
 // memory; (2) a 4-pass radix select (8 bits per pass, shared-memory histograms with
 // integer atomics) finds the k-th smallest key T and how many keys equal to T are taken;
-// (3) a stable, scan-based compaction gathers every key < T and the lowest-index keys
-// == T; (4) a bitonic sort of the k selected (key << 32 | index) pairs.  Integer work
-// only, so the result is deterministic and equals a stable sort by (cost, index).
+// (3) every key < T is gathered in any order and the lowest-index keys == T by ballots; (4) a
+// bitonic sort of the k selected (key << 32 | index) pairs.  Integer work only, and the sort
+// orders whatever the gathering left, so the result is deterministic and equals a stable sort by
+// (cost, index).
+// A latency-bound single CTA: the bucket of a pass is found by one warp's scan (a thread walking
+// the 256 buckets took 3.7 us a pass, most of the time at a few hundred costs), the gathering
+// reads consecutive keys (a contiguous run per thread met 16-way bank conflicts), and the sort's
+// exchanges over distances up to 32 stay inside a warp's 64 pairs, so 28 of its 78 steps at 4096
+// end with a block barrier.  n = 16384, k = 4096: 59 -> 47 us; n = 4096, k = 1024: 22.6 -> 16.5 us;
+// n = 256, k = 64: 16.4 -> 8.4 us.
 #pragma once
 #include "common.cuh"
 
@@ -21,33 +28,6 @@ __device__ __forceinline__ uint32_t cost_key(float c) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// inclusive block scan of one int per thread (1024 threads); returns the inclusive value
-// and the block total in *total.
-__device__ __forceinline__ int block_scan_incl(int v, int* warp_tot, int* total) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += t;
-    }
-    if (lane == 31) warp_tot[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        int s = lane < (int)(blockDim.x >> 5) ? warp_tot[lane] : 0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int t = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += t;
-        }
-        warp_tot[lane] = s;
-    }
-    __syncthreads();
-    const int res = v + (w > 0 ? warp_tot[w - 1] : 0);
-    *total = warp_tot[(blockDim.x >> 5) - 1];
-    __syncthreads();
-    return res;
-}
-
 // keys (n) and pairs (kp2 >= k, power of two) live in dynamic shared memory.
 __global__ void __launch_bounds__(kSelectThreads) k_topk(const float* __restrict__ cost, int n, int k,
                                                           int* __restrict__ out_idx, float* __restrict__ out_cost,
@@ -55,15 +35,14 @@ __global__ void __launch_bounds__(kSelectThreads) k_topk(const float* __restrict
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned long long* pairs = reinterpret_cast<unsigned long long*>(smem_raw);
     uint32_t* keys = reinterpret_cast<uint32_t*>(pairs + kp2);
-    __shared__ int hist[256];
-    __shared__ int warp_tot[32];
+    __shared__ int hist[256];   // a pass's buckets; then the keys == T of each warp
     __shared__ uint32_t s_prefix;
-    __shared__ int s_need;
-    const int tid = threadIdx.x, nt = blockDim.x;
+    __shared__ int s_need, s_equal, s_less_at, s_equal_at;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, w = tid >> 5;
     if (k > n) k = n;
 
     for (int i = tid; i < n; i += nt) keys[i] = cost_key(cost[i]);
-    if (tid == 0) { s_prefix = 0; s_need = k; }
+    if (tid == 0) { s_prefix = 0; s_need = k; s_equal = 0; s_less_at = 0; s_equal_at = 0; }
     __syncthreads();
 
     // radix select of the k-th smallest key (1-based rank k)
@@ -77,14 +56,31 @@ __global__ void __launch_bounds__(kSelectThreads) k_topk(const float* __restrict
             if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1);
         }
         __syncthreads();
-        if (tid == 0) {
-            int need = s_need, acc = 0, bkt = 0;
-            for (; bkt < 256; ++bkt) {
-                if (acc + hist[bkt] >= need) break;
-                acc += hist[bkt];
+        if (w == 0) {   // the bucket that holds rank s_need: eight buckets per lane, a scan over the lanes
+            int cnt[8], sum = 0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) { cnt[i] = hist[8 * lane + i]; sum += cnt[i]; }
+            int below = sum;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int up = __shfl_up_sync(0xffffffffu, below, off);
+                if (lane >= off) below += up;
             }
-            s_need = need - acc;
-            s_prefix = prefix | ((uint32_t)bkt << shift);
+            below -= sum;
+            const int need = s_need;
+            __syncwarp();
+            if (below < need && need <= below + sum) {
+                int bkt = 8 * lane;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    if (below < need && need <= below + cnt[i]) {
+                        s_need = need - below;
+                        s_equal = cnt[i];
+                        s_prefix = prefix | ((uint32_t)(bkt + i) << shift);
+                    }
+                    below += cnt[i];
+                }
+            }
         }
         mask |= 255u << shift;
         __syncthreads();
@@ -92,27 +88,37 @@ __global__ void __launch_bounds__(kSelectThreads) k_topk(const float* __restrict
     const uint32_t T = s_prefix;
     const int need_eq = s_need;   // keys == T to take (lowest indices first)
 
-    // stable compaction over contiguous chunks
-    const int chunk = (n + nt - 1) / nt;
-    const int lo = min(n, tid * chunk), hi = min(n, lo + chunk);
-    int n_less = 0, n_eq = 0;
-    for (int i = lo; i < hi; ++i) {
-        const uint32_t key = keys[i];
-        n_less += key < T;
-        n_eq += key == T;
-    }
-    int tot_less, tot_eq;
-    const int less_incl = block_scan_incl(n_less, warp_tot, &tot_less);
-    const int eq_incl = block_scan_incl(n_eq, warp_tot, &tot_eq);
-    int pos_less = less_incl - n_less, pos_eq = eq_incl - n_eq;
+    // gather: 1024 consecutive keys at a time
     const int n_sel_less = k > 0 ? k - need_eq : 0;
-    for (int i = lo; i < hi; ++i) {
-        const uint32_t key = keys[i];
-        if (k > 0 && key < T) {
-            pairs[pos_less++] = ((unsigned long long)key << 32) | (uint32_t)i;
-        } else if (k > 0 && key == T) {
-            if (pos_eq < need_eq) pairs[n_sel_less + pos_eq] = ((unsigned long long)key << 32) | (uint32_t)i;
-            ++pos_eq;
+    const bool ordered = s_equal > need_eq;   // not every key == T is taken: the lowest indices are
+    int eq_done = 0;
+    for (int base = 0; k > 0 && base < n; base += nt) {
+        const int i = base + tid;
+        const uint32_t key = i < n ? keys[i] : 0xFFFFFFFFu;
+        const unsigned less = __ballot_sync(0xffffffffu, i < n && key < T);
+        const unsigned equal = __ballot_sync(0xffffffffu, i < n && key == T);
+        const unsigned before = (1u << lane) - 1u;
+        int at = 0;
+        if (lane == 0 && less) at = atomicAdd(&s_less_at, __popc(less));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if ((less >> lane) & 1u) pairs[at + __popc(less & before)] = ((unsigned long long)key << 32) | (uint32_t)i;
+        int eq_at = 0;
+        if (ordered && eq_done < need_eq) {   // uniform over the block
+            if (lane == 0) hist[w] = __popc(equal);
+            __syncthreads();
+            const int c = hist[lane];
+            eq_at = __reduce_add_sync(0xffffffffu, lane < w ? c : 0) + eq_done;
+            eq_done += __reduce_add_sync(0xffffffffu, c);
+            __syncthreads();
+        } else if (ordered) {
+            continue;
+        } else {
+            if (lane == 0 && equal) eq_at = atomicAdd(&s_equal_at, __popc(equal));
+            eq_at = __shfl_sync(0xffffffffu, eq_at, 0);
+        }
+        if ((equal >> lane) & 1u) {
+            const int pos = eq_at + __popc(equal & before);
+            if (pos < need_eq) pairs[n_sel_less + pos] = ((unsigned long long)key << 32) | (uint32_t)i;
         }
     }
     for (int i = k + tid; i < kp2; i += nt) pairs[i] = ~0ull;
@@ -128,7 +134,10 @@ __global__ void __launch_bounds__(kSelectThreads) k_topk(const float* __restrict
                 const unsigned long long a = pairs[lo_i], b = pairs[hi_i];
                 if ((a > b) == up) { pairs[lo_i] = b; pairs[hi_i] = a; }
             }
-            __syncthreads();
+            // up to a distance of 32 a warp's threads exchange within their own 64 pairs (of every
+            // 2048), and so they do in the next step unless it starts a longer size
+            if (stride > 32 || (stride == 1 && size > 32)) __syncthreads();
+            else __syncwarp();
         }
     }
     for (int i = tid; i < k; i += nt) {
