@@ -175,6 +175,30 @@ __device__ __forceinline__ float warp_fmax(float v) {
     return r;
 }
 
+// Sums of N values per lane over the warp by recursive halving: at the step of lane bit `off` a
+// lane keeps the half of its values selected by that bit and adds the partner's copy of it; the
+// remaining exchanges complete the sum.  Lane L ends with the sum of value (top log2 N bits of L),
+// added up in the pairing of warp_sum (bits 16, 8, 4, 2, 1), hence the same bits, in N - 1 + 5 -
+// log2 N shuffles in place of 5 N.
+template <int N>
+__device__ __forceinline__ float warp_sums(float v[N]) {
+    const int lane = threadIdx.x & 31;
+    int off = 16;
+#pragma unroll
+    for (int half = N / 2; half >= 1; half >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const float send = up ? v[i] : v[i + half], keep = up ? v[i + half] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+        off >>= 1;
+    }
+#pragma unroll
+    for (; off >= 1; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+    return v[0];
+}
+
 // ------------------------------------------------------------------------------ geometry
 // Penetration of sphere (c, r) into a cuboid, pen = max(0, -sd) with
 //   p = R^T (c - centre), q = |p| - h,  sd = ||max(q,0)|| + min(max_k q_k, 0) - r.

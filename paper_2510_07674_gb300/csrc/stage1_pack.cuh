@@ -13,6 +13,12 @@
 // cube's sphere-side gradient is reduced inside its lane group and stored once per
 // evaluation (gcell); lanes < B then add their cubes in order, so sums are deterministic.
 // The cube side of a block pair is reduced over the warp once per lower block.
+//
+// Bound by instruction issue.  The 32 spheres of a pass (four cubes) meet the cubes below whose boxes
+// they reach: one ballot per 32 cubes, in the order of the cubes, so the sums stay those of all of them.
+// The cubes' boxes are laid out once per evaluation: 32 lanes that index the constant bank by cube in
+// every pass cost more than the cull saves (4.88 -> 5.26 ms).  A handful of walls is tested without a
+// cull, which costs as much as they do.  Descending 4096 packings of 8 blocks: 4.88 -> 4.30 ms.
 #pragma once
 #include "stage1.cuh"
 
@@ -21,7 +27,8 @@ namespace spasm {
 __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const float4* __restrict__ cub, int n_cub,
                                                      const float4* __restrict__ osph, int n_osph, const float* x,
                                                      bool quad, int mode, const float* b_in, float s_coll_in,
-                                                     float* g, PlaceScratch& ps, float4* gcell, PlaceOut& out) {
+                                                     float* g, PlaceScratch& ps, float4* gcell, float4* cube,
+                                                     PlaceOut* out) {
     const int lane = threadIdx.x & 31;
     const int B = sc.B;
     const bool want_grad = mode != kPlaceForward;
@@ -38,6 +45,14 @@ __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const fl
             const float b = mode == kPlaceStage1 ? sc.w_height * (my_e > 0.f ? 1.f : (my_e < 0.f ? -1.f : 0.f)) : b_in[i];
             g[4 * i] = 0.f; g[4 * i + 1] = 0.f; g[4 * i + 2] = b; g[4 * i + 3] = 0.f;
         }
+    }
+    __syncwarp();
+    for (int k = lane; k < sc.n_cells; k += 32) {
+        const int i = sc.cell_block[k];
+        const float2 off = sc.cell[k];
+        const float ci = ps.bc[i][1].x, si = ps.bc[i][1].y;
+        cube[k] = make_float4(x[4 * i] + ci * off.x - si * off.y, x[4 * i + 1] + si * off.x + ci * off.y, x[4 * i + 2],
+                              (fabsf(ci) + fabsf(si)) * half.x);
     }
     __syncwarp();
 
@@ -78,8 +93,23 @@ __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const fl
                 }
             }
         }
-        // cubes of the blocks below j in the skeleton order
-        for (int i = 0; i + 1 < B; ++i) {
+        // cubes of the blocks below j in the skeleton order, those near the 32 spheres of this pass
+        const SphereBox sb = warp_sphere_box(valid, cx, cy, cz, r);
+        unsigned long long near_cubes = 0ull;
+        for (int first = 0; first < sc.n_cells; first += 32) {
+            bool near_cube = false;
+            if (first + lane < sc.n_cells) {
+                const float4 q = cube[first + lane];
+                near_cube = sb.near_box(q.x, q.y, q.z, q.w, q.w, half.z);
+            }
+            near_cubes |= (unsigned long long)__ballot_sync(0xffffffffu, near_cube) << first;
+        }
+        const int j_top = sc.cell_block[min(base + 31, n_items - 1) >> 3];   // cells are in block order
+        near_cubes &= (1ull << sc.cell_start[j_top]) - 1ull;                // cell_start[j_top] < kMaxCells
+        while (near_cubes) {
+            const int i = sc.cell_block[__ffsll((long long)near_cubes) - 1];
+            unsigned long long cubes = near_cubes & ((1ull << sc.cell_start[i + 1]) - 1ull);   // of block i
+            near_cubes ^= cubes;
             float bx = 0.f, by = 0.f, bz = 0.f, byaw = 0.f;   // dC/d(pose i) from this sphere
             bool hit = false;
             const float oxi = x[4 * i], oyi = x[4 * i + 1], ozi = x[4 * i + 2];
@@ -88,7 +118,8 @@ __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const fl
                 const float ci = ps.bc[i][1].x, si = ps.bc[i][1].y;
                 const float4 c0 = make_float4(ci, si, 0.f, half.x), c1 = make_float4(-si, ci, 0.f, half.y);
                 const float4 c2 = make_float4(0.f, 0.f, 1.f, half.z);
-                for (int kk = sc.cell_start[i]; kk < sc.cell_start[i + 1]; ++kk) {
+                for (; cubes; cubes &= cubes - 1ull) {
+                    const int kk = __ffsll((long long)cubes) - 1;
                     const float2 off = sc.cell[kk];
                     const float4 o = make_float4(oxi + ci * off.x - si * off.y, oyi + si * off.x + ci * off.y, ozi, 0.f);
                     float gx, gy, gz;
@@ -107,24 +138,16 @@ __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const fl
                 }
             }
             if (want_grad && __any_sync(0xffffffffu, hit)) {
-                bx = warp_sum(bx); by = warp_sum(by); bz = warp_sum(bz); byaw = warp_sum(byaw);
-                if (lane == 0) {
-                    g[4 * i] += s_coll * bx; g[4 * i + 1] += s_coll * by;
-                    g[4 * i + 2] += s_coll * bz; g[4 * i + 3] += s_coll * byaw;
-                }
+                float d4[4] = {bx, by, bz, byaw};
+                const float d = warp_sums<4>(d4);   // lane 8 n: value n
+                if ((lane & 7) == 0) g[4 * i + (lane >> 3)] += s_coll * d;
                 __syncwarp();
             }
         }
         if (want_grad) {
-            float gyaw = ax * (-s * lx - c * ly) + ay * (c * lx - s * ly);   // dc/dyaw_j
-#pragma unroll
-            for (int off = 4; off > 0; off >>= 1) {
-                ax += __shfl_xor_sync(0xffffffffu, ax, off);
-                ay += __shfl_xor_sync(0xffffffffu, ay, off);
-                az += __shfl_xor_sync(0xffffffffu, az, off);
-                gyaw += __shfl_xor_sync(0xffffffffu, gyaw, off);
-            }
-            if (valid && m == 0) gcell[k] = make_float4(ax, ay, az, gyaw);
+            const float gyaw = ax * (-s * lx - c * ly) + ay * (c * lx - s * ly);   // dc/dyaw_j
+            const float d = group_sums(ax, ay, az, gyaw);
+            if (valid && (m & 1) == 0) reinterpret_cast<float*>(gcell + k)[m >> 1] = d;
         }
     }
     __syncwarp();
@@ -137,22 +160,24 @@ __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const fl
         }
         g[4 * i] += s_coll * sx; g[4 * i + 1] += s_coll * sy; g[4 * i + 2] += s_coll * sz; g[4 * i + 3] += s_coll * syaw;
     }
-    out.c_coll = warp_sum(coll);
-    out.maxpen = warp_max(maxpen);
-    out.c_stable = 0.f;
-    out.c_height = warp_sum(lane < B ? fabsf(my_e) : 0.f);
-    out.maxD = 0.f;
-    out.maxdz = warp_max(lane < B ? fabsf(my_e) : 0.f);
+    if (out) {
+        out->c_coll = warp_sum(coll);
+        out->maxpen = warp_max(maxpen);
+        out->c_stable = 0.f;
+        out->c_height = warp_sum(lane < B ? fabsf(my_e) : 0.f);
+        out->maxD = 0.f;
+        out->maxdz = warp_max(lane < B ? fabsf(my_e) : 0.f);
+    }
     __syncwarp();
 }
 
 // The placement cost of the problem's goal (tower or packing).
 __device__ __forceinline__ void place_eval(const Scalars& sc, const float4* __restrict__ cub, int n_cub,
                                            const float4* __restrict__ osph, int n_osph, const float* x, bool quad,
-                                           int mode, float* g, PlaceScratch& ps, float4* gcell, uint32_t* cand,
-                                           PlaceOut& out) {
+                                           int mode, float* g, PlaceScratch& ps, float4* gcell, float4* cube,
+                                           uint32_t* cand, PlaceOut* out) {
     if (sc.kind == kKindPack)
-        place_eval_pack_warp(sc, cub, n_cub, osph, n_osph, x, quad, mode, nullptr, 0.f, g, ps, gcell, out);
+        place_eval_pack_warp(sc, cub, n_cub, osph, n_osph, x, quad, mode, nullptr, 0.f, g, ps, gcell, cube, out);
     else
         place_eval_warp(sc, cub, n_cub, osph, n_osph, x, quad, mode, nullptr, nullptr, 0.f, g, ps, cand, out);
 }
