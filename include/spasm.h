@@ -403,7 +403,8 @@ spasm_status spasm_reset_stats(spasm_problem_t problem);
  * stream (not the legacy default stream: the batch is captured as CUDA graphs).  The first
  * attempt of stage 1 of every problem not yet placed runs as one graph; stage 2 of every
  * placed problem (lift, one persistent launch of the trajectory kernel over the particles
- * of all problems, selection, FP64 check) runs as a second graph.  A problem that needs
+ * of all problems, or one per launch shape where the shape is left to the library, selection,
+ * FP64 check) runs as a second graph.  A problem that needs
  * further attempts continues alone on its own stream, as spasm_optimize would.  Each
  * problem's outcome is then read with spasm_result, and equals what spasm_optimize gives
  * (the same arithmetic for every particle, whatever the schedule).  Returns SPASM_OK unless
@@ -442,8 +443,8 @@ spasm_status spasm_batch_autotune(spasm_problem_t* problems, int n, void* cuda_s
  * memory (spasm_problem_bytes) fits budget_bytes (a request larger than the whole budget is
  * admitted when nothing else is in flight), created on the scheduler's stream of the device
  * current at creation, and their stage 1 runs (with its device-side attempt loop); then one
- * persistent launch of the trajectory kernel runs the descent of the particles of every
- * request in flight, followed per request by its satisfying selection, its attempt decision
+ * persistent launch of the trajectory kernel per launch shape (one or two) runs the descent of the
+ * particles of every request in flight, followed per request by its satisfying selection, its attempt decision
  * and the FP64 check; requests that finished retire, the others re-lift with their next
  * attempt counter for the next epoch.  A request that arrives during an epoch joins at the
  * next one.  Each request's result is the one spasm_optimize gives for it, whatever else is in

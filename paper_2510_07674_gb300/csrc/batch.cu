@@ -2,7 +2,8 @@
 // for many independent problems).  One CUDA graph holds the whole batch: stage 1 of every
 // problem not yet placed (each with its own device-side attempt loop, in parallel branches),
 // the first stage-2 lift of every problem, one persistent launch of the trajectory kernel
-// over the particles of all problems, then per problem (in parallel branches) the
+// over the particles of all problems (two side by side, one per launch shape, where the shape is
+// left to the library and the problems differ in the better one), then per problem (in parallel branches) the
 // satisfying selection, its device-side re-lift loop and the FP64 check.  Every particle
 // runs the same arithmetic as in the single-problem launches, so each problem's result
 // equals its spasm_optimize result.

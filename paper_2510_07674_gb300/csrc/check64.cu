@@ -15,7 +15,8 @@
 //                   is penetrated), a warp per configuration; usually one or two of 620.
 // The margin bounds the FP32 evaluation's error (Scalars64::margin, some hundred rounding steps of
 // the scene's extent), so the configuration that holds the FP64 maximum is always among those
-// repeated, and the metrics are those of the full FP64 evaluation: 41 us for the same 32.
+// repeated, and the metrics are those of the full FP64 evaluation: 85 us for the same 32 (the
+// screen 55, beside the FP64 metrics' latency, the second pass 31).
 // Joints too large for an FP32 angle, or NaN, are repeated always.
 #include "check64.h"
 #include "stage2.cuh"

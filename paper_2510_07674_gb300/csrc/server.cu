@@ -7,15 +7,16 @@
 //      request larger than the whole budget is admitted when nothing else is in flight;
 //   2. create each admitted request's problem and enqueue its stage 1 (the graph with the
 //      device-side attempt loop of spasm_place) and its first lift;
-//   3. one persistent launch of the trajectory kernel over the particles of every request in
-//      flight (a shared work list of particle runs, gated per request by its placement count);
+//   3. one persistent launch of the trajectory kernel per launch shape (one or two, side by side)
+//      over the particles of every request in flight (a shared work list of particle runs, gated
+//      per request by its placement count);
 //   4. per request: the satisfying selection and the attempt decision on the device, and the
 //      FP64 check of the best P;
 //   5. one host wait, then retire the requests that finished (results copied to the host,
 //      problems destroyed, budget returned) and re-lift the others with their next attempt
 //      counter for the next epoch.
-// Requests that arrive during an epoch join at the next one, so the GPU runs one launch over
-// all work in flight rather than one solve per request.  Every particle runs the code of a
+// Requests that arrive during an epoch join at the next one, so the GPU runs
+// all work in flight together rather than one solve per request.  Every particle runs the code of a
 // single solve with the same Philox streams, so a request's result does not depend on what
 // else is in flight.  Host waits are bounded; a request is cancelled while it is queued, or
 // at the next epoch boundary while it is in flight.
