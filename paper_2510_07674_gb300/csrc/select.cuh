@@ -9,10 +9,12 @@
 // (cost, index).
 // A latency-bound single CTA: the bucket of a pass is found by one warp's scan (a thread walking
 // the 256 buckets took 3.7 us a pass, most of the time at a few hundred costs), the gathering
-// reads consecutive keys (a contiguous run per thread met 16-way bank conflicts), and the sort's
-// exchanges over distances up to 32 stay inside a warp's 64 pairs, so 28 of its 78 steps at 4096
-// end with a block barrier.  n = 16384, k = 4096: 59 -> 47 us; n = 4096, k = 1024: 22.6 -> 16.5 us;
-// n = 256, k = 64: 16.4 -> 8.4 us.
+// reads consecutive keys (a contiguous run per thread met 16-way bank conflicts), and the sort
+// keeps the pairs in registers: 63 of its 78 steps at 4096 stay inside a thread or a warp, the
+// other 15 take nine passes through shared memory (every step through shared memory: 27 us at
+// 4096 pairs, 10 us now).  n = 16384, k = 4096: 59.5 -> 30.8 us, of which the four passes over the
+// keys 11 and the launch with its latency 8; n = 4096, k = 1024: 22.6 -> 14.4 us; n = 256, k = 64:
+// 16.4 -> 8.2 us.
 #pragma once
 #include "common.cuh"
 
@@ -28,7 +30,91 @@ __device__ __forceinline__ uint32_t cost_key(float c) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// keys (n) and pairs (kp2 >= k, power of two) live in dynamic shared memory.
+// Bitonic sort of kp2 pairs (ascending, a power of two; kp2 <= 1024 for E = 1, else kp2 = 1024 E) by the whole
+// block.  Thread t keeps pairs t E .. t E + E - 1 in registers: exchanges over distances below E stay in the
+// thread, below 32 E in the warp (shuffles); the longer ones go through shared memory two distances at a
+// time, a barrier per pair of distances.  Leaves the sorted pairs in v (all ones beyond kp2).
+template <int E>
+__device__ __forceinline__ void sort_pairs(unsigned long long* pairs, int kp2, unsigned long long (&v)[E]) {
+    const int t = threadIdx.x, nt = blockDim.x, total = kp2 < 32 ? 32 : kp2;
+    const bool mine = t * E < total;   // uniform over a warp
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = t * E + e < kp2 ? pairs[t * E + e] : ~0ull;
+    for (int size = 2; size <= total; size <<= 1) {
+        int stride = size >> 1;
+        if (stride >= 32 * E) {
+            if (mine)
+#pragma unroll
+                for (int e = 0; e < E; ++e) pairs[t * E + e] = v[e];
+            __syncthreads();
+            for (; stride >= 64 * E; stride >>= 2) {
+                const int half = stride >> 1;
+                for (int i = t; i < total / 4; i += nt) {
+                    const int base = 4 * i - 3 * (i & (half - 1));
+                    const bool up = (base & size) == 0;
+                    unsigned long long a = pairs[base], b = pairs[base + half];
+                    unsigned long long c = pairs[base + stride], d = pairs[base + stride + half], x;
+                    if ((a > c) == up) { x = a; a = c; c = x; }
+                    if ((b > d) == up) { x = b; b = d; d = x; }
+                    if ((a > b) == up) { x = a; a = b; b = x; }
+                    if ((c > d) == up) { x = c; c = d; d = x; }
+                    pairs[base] = a; pairs[base + half] = b;
+                    pairs[base + stride] = c; pairs[base + stride + half] = d;
+                }
+                __syncthreads();
+            }
+            if (stride == 32 * E) {
+                for (int i = t; i < total / 2; i += nt) {
+                    const int lo = 2 * i - (i & (stride - 1)), hi = lo + stride;
+                    const unsigned long long a = pairs[lo], b = pairs[hi];
+                    if ((a > b) == ((lo & size) == 0)) { pairs[lo] = b; pairs[hi] = a; }
+                }
+                __syncthreads();
+                stride >>= 1;
+            }
+            if (mine)
+#pragma unroll
+                for (int e = 0; e < E; ++e) v[e] = pairs[t * E + e];
+        }
+        if (!mine) continue;
+        for (; stride >= E; stride >>= 1) {
+            const int lanes = stride / E;
+            const bool keep_min = ((t & lanes) == 0) == (((t * E) & size) == 0);
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const unsigned long long o = __shfl_xor_sync(0xffffffffu, v[e], lanes);
+                if ((o < v[e]) == keep_min) v[e] = o;
+            }
+        }
+#pragma unroll
+        for (int st = E / 2; st > 0; st >>= 1) {
+            if (st > stride) continue;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                if (e & st) continue;
+                const unsigned long long a = v[e], b = v[e + st];
+                if ((a > b) == (((t * E + e) & size) == 0)) { v[e] = b; v[e + st] = a; }
+            }
+        }
+    }
+}
+
+template <int E>
+__device__ __forceinline__ void sort_and_write(unsigned long long* pairs, int kp2, int k, const float* __restrict__ cost,
+                                               int* __restrict__ out_idx, float* __restrict__ out_cost) {
+    unsigned long long v[E];
+    sort_pairs<E>(pairs, kp2, v);
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int i = (int)threadIdx.x * E + e;
+        if (i >= k) continue;
+        const int idx = (int)(uint32_t)(v[e] & 0xffffffffull);
+        out_idx[i] = idx;
+        if (out_cost) out_cost[i] = cost[idx];
+    }
+}
+
+// keys (n) and pairs (kp2 >= k, power of two) live in dynamic shared memory; kp2 <= 8192.
 __global__ void __launch_bounds__(kSelectThreads) k_topk(const float* __restrict__ cost, int n, int k,
                                                           int* __restrict__ out_idx, float* __restrict__ out_cost,
                                                           int kp2) {
@@ -124,27 +210,10 @@ __global__ void __launch_bounds__(kSelectThreads) k_topk(const float* __restrict
     for (int i = k + tid; i < kp2; i += nt) pairs[i] = ~0ull;
     __syncthreads();
 
-    // bitonic sort of kp2 pairs (ascending)
-    for (int size = 2; size <= kp2; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = tid; i < kp2 / 2; i += nt) {
-                const int lo_i = 2 * i - (i & (stride - 1));
-                const int hi_i = lo_i + stride;
-                const bool up = (lo_i & size) == 0;
-                const unsigned long long a = pairs[lo_i], b = pairs[hi_i];
-                if ((a > b) == up) { pairs[lo_i] = b; pairs[hi_i] = a; }
-            }
-            // up to a distance of 32 a warp's threads exchange within their own 64 pairs (of every
-            // 2048), and so they do in the next step unless it starts a longer size
-            if (stride > 32 || (stride == 1 && size > 32)) __syncthreads();
-            else __syncwarp();
-        }
-    }
-    for (int i = tid; i < k; i += nt) {
-        const int idx = (int)(uint32_t)(pairs[i] & 0xffffffffull);
-        out_idx[i] = idx;
-        if (out_cost) out_cost[i] = cost[idx];
-    }
+    if (kp2 <= 1024) sort_and_write<1>(pairs, kp2, k, cost, out_idx, out_cost);
+    else if (kp2 == 2048) sort_and_write<2>(pairs, kp2, k, cost, out_idx, out_cost);
+    else if (kp2 == 4096) sort_and_write<4>(pairs, kp2, k, cost, out_idx, out_cost);
+    else sort_and_write<8>(pairs, kp2, k, cost, out_idx, out_cost);   // 8192
 }
 
 }  // namespace spasm
