@@ -19,32 +19,47 @@ struct S1Warp {
     uint32_t cand[kMaxCub / 32 + kMaxOSph / 32];   // candidate obstacles of the particle (tower goal)
 };
 
-// dynamic shared memory: mbarrier | env cuboids | env spheres | per-warp scratch
+// dynamic shared memory: mbarrier | env cuboids | env spheres | boxes of the packing's walls | per-warp scratch
 __host__ __device__ inline size_t s1_env_offset() { return 16; }
-__host__ __device__ inline size_t s1_warp_offset(int n_cub, int n_osph) {
-    size_t off = 16 + (size_t)n_cub * 64 + (size_t)n_osph * 16;
-    return (off + 15) & ~(size_t)15;
+__host__ __device__ inline size_t s1_wall_offset(const Scalars& sc) {
+    return 16 + (size_t)sc.n_cub * 64 + (size_t)sc.n_osph * 16;
 }
-static size_t s1_smem_bytes(const Scalars& sc) {
-    return s1_warp_offset(sc.n_cub, sc.n_osph) + sizeof(S1Warp) * kS1Warps;
+__host__ __device__ inline size_t s1_warp_offset(const Scalars& sc) {
+    return s1_wall_offset(sc) + (sc.kind == kKindPack ? (size_t)sc.n_cub * 32 : 0);
 }
+static size_t s1_smem_bytes(const Scalars& sc) { return s1_warp_offset(sc) + sizeof(S1Warp) * kS1Warps; }
 
 struct S1Smem {
     uint64_t* bar;
     float4* cub;
     float4* osph;
+    float4* wall;
     S1Warp* warp;
 };
 
+template <bool kTower>
 __device__ __forceinline__ bool s1_setup(const Scalars& sc, DevTables t, S1Smem& s, int* err) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     s.bar = reinterpret_cast<uint64_t*>(smem_raw);
     s.cub = reinterpret_cast<float4*>(smem_raw + s1_env_offset());
     s.osph = s.cub + 4 * sc.n_cub;
-    s.warp = reinterpret_cast<S1Warp*>(smem_raw + s1_warp_offset(sc.n_cub, sc.n_osph));
-    return stage_tables(s.cub, t.cub, (uint32_t)sc.n_cub * 64u, s.osph, t.osph, (uint32_t)sc.n_osph * 16u, s.bar, err);
+    s.wall = reinterpret_cast<float4*>(smem_raw + s1_wall_offset(sc));
+    s.warp = reinterpret_cast<S1Warp*>(smem_raw + s1_warp_offset(sc));
+    const bool staged = stage_tables(s.cub, t.cub, (uint32_t)sc.n_cub * 64u, s.osph, t.osph, (uint32_t)sc.n_osph * 16u, s.bar, err);
+    if (!kTower && staged && sc.kind == kKindPack) {
+        for (int o = threadIdx.x; o < sc.n_cub; o += kS1Threads) {
+            const float4 c0 = s.cub[4 * o], c1 = s.cub[4 * o + 1], c2 = s.cub[4 * o + 2], c3 = s.cub[4 * o + 3];
+            s.wall[2 * o] = c0;
+            s.wall[2 * o + 1] = make_float4(fabsf(c1.x) * c1.w + fabsf(c2.x) * c2.w + fabsf(c3.x) * c3.w,
+                                            fabsf(c1.y) * c1.w + fabsf(c2.y) * c2.w + fabsf(c3.y) * c3.w,
+                                            fabsf(c1.z) * c1.w + fabsf(c2.z) * c2.w + fabsf(c3.z) * c3.w, 0.f);
+        }
+        __syncthreads();
+    }
+    return staged;
 }
 
+template <bool kTower>
 __global__ void __launch_bounds__(kS1Threads) k_place_sample_cost(const __grid_constant__ Scalars sc, DevTables t, int n,
                                                                    uint32_t attempt, float* __restrict__ x_out,
                                                                    float* __restrict__ cost_out, int* err,
@@ -52,7 +67,7 @@ __global__ void __launch_bounds__(kS1Threads) k_place_sample_cost(const __grid_c
     uint64_t key = sc.seed;   // the Philox key
     if (ctl) { attempt = ctl->attempt; key = ctl->seed; }
     S1Smem s;
-    if (!s1_setup(sc, t, s, err)) return;
+    if (!s1_setup<kTower>(sc, t, s, err)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int p = blockIdx.x * kS1Warps + w;
     if (p >= n) return;
@@ -68,19 +83,20 @@ __global__ void __launch_bounds__(kS1Threads) k_place_sample_cost(const __grid_c
     }
     __syncwarp();
     PlaceOut o;
-    place_eval(sc, s.cub, sc.n_cub, s.osph, sc.n_osph, W.x, false, kPlaceForward, nullptr, W.ps,
+    place_eval<kTower>(sc, s.cub, s.wall, sc.n_cub, s.osph, sc.n_osph, W.x, false, kPlaceForward, nullptr, W.ps,
                W.gcell, W.cube, W.cand, &o);
     for (int v = lane; v < 4 * sc.B; v += 32) x_out[(size_t)v * n + p] = W.x[v];
     if (lane == 0) cost_out[p] = place_cost_value(sc, o);
 }
 
+template <bool kTower>
 __global__ void __launch_bounds__(kS1Threads) k_place_eval(const __grid_constant__ Scalars sc, DevTables t, int n,
                                                             const float* __restrict__ x, int quad,
                                                             float* __restrict__ cost, float* __restrict__ grad,
                                                             float* __restrict__ metrics, float* __restrict__ terms,
                                                             int* err) {
     S1Smem s;
-    if (!s1_setup(sc, t, s, err)) return;
+    if (!s1_setup<kTower>(sc, t, s, err)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int p = blockIdx.x * kS1Warps + w;
     if (p >= n) return;
@@ -88,7 +104,7 @@ __global__ void __launch_bounds__(kS1Threads) k_place_eval(const __grid_constant
     for (int v = lane; v < 4 * sc.B; v += 32) W.x[v] = x[(size_t)v * n + p];
     __syncwarp();
     PlaceOut o;
-    place_eval(sc, s.cub, sc.n_cub, s.osph, sc.n_osph, W.x, quad != 0, grad ? kPlaceStage1 : kPlaceForward, W.g, W.ps,
+    place_eval<kTower>(sc, s.cub, s.wall, sc.n_cub, s.osph, sc.n_osph, W.x, quad != 0, grad ? kPlaceStage1 : kPlaceForward, W.g, W.ps,
                W.gcell, W.cube, W.cand, &o);
     if (grad)
         for (int v = lane; v < 4 * sc.B; v += 32) grad[(size_t)v * n + p] = W.g[v];
@@ -102,14 +118,15 @@ __global__ void __launch_bounds__(kS1Threads) k_place_eval(const __grid_constant
 // Alg. 1, linear cost descent (eta = eta_init (1 - k/K_lin)) then quadratic refinement
 // (fixed alpha), each followed by the box projection; then GetSatisfyingParticles and
 // the final (quadratic-form) cost.  The whole loop runs inside one launch.
-__global__ void __launch_bounds__(kS1Threads) k_place_descend(const __grid_constant__ Scalars sc, DevTables t, int m,
+template <bool kTower>
+__global__ void __launch_bounds__(kS1Threads, 4) k_place_descend(const __grid_constant__ Scalars sc, DevTables t, int m,
                                                                const float* __restrict__ x_src, int ld_src,
                                                                const int* __restrict__ idx, float* __restrict__ x_dst,
                                                                int k_lin, int k_quad, float* __restrict__ cost,
                                                                int* __restrict__ sat, float* __restrict__ metrics,
                                                                int* err) {
     S1Smem s;
-    if (!s1_setup(sc, t, s, err)) return;
+    if (!s1_setup<kTower>(sc, t, s, err)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int p = blockIdx.x * kS1Warps + w;
     if (p >= m) return;
@@ -121,18 +138,18 @@ __global__ void __launch_bounds__(kS1Threads) k_place_descend(const __grid_const
     PlaceOut o;
     for (int k = 1; k <= k_lin; ++k) {
         const float eta = sc.eta_init * (1.f - (float)k / (float)k_lin);
-        place_eval(sc, s.cub, sc.n_cub, s.osph, sc.n_osph, W.x, false, kPlaceStage1, W.g, W.ps,
+        place_eval<kTower>(sc, s.cub, s.wall, sc.n_cub, s.osph, sc.n_osph, W.x, false, kPlaceStage1, W.g, W.ps,
                W.gcell, W.cube, W.cand, nullptr);
         for (int v = lane; v < nv; v += 32) W.x[v] = place_clamp(sc, v, W.x[v] - eta * W.g[v]);
         __syncwarp();
     }
     for (int k = 1; k <= k_quad; ++k) {
-        place_eval(sc, s.cub, sc.n_cub, s.osph, sc.n_osph, W.x, true, kPlaceStage1, W.g, W.ps,
+        place_eval<kTower>(sc, s.cub, s.wall, sc.n_cub, s.osph, sc.n_osph, W.x, true, kPlaceStage1, W.g, W.ps,
                W.gcell, W.cube, W.cand, nullptr);
         for (int v = lane; v < nv; v += 32) W.x[v] = place_clamp(sc, v, W.x[v] - sc.alpha * W.g[v]);
         __syncwarp();
     }
-    place_eval(sc, s.cub, sc.n_cub, s.osph, sc.n_osph, W.x, true, kPlaceForward, nullptr, W.ps,
+    place_eval<kTower>(sc, s.cub, s.wall, sc.n_cub, s.osph, sc.n_osph, W.x, true, kPlaceForward, nullptr, W.ps,
                W.gcell, W.cube, W.cand, &o);
     for (int v = lane; v < nv; v += 32) x_dst[(size_t)v * m + p] = W.x[v];
     if (lane == 0) {
@@ -168,44 +185,36 @@ __global__ void k_gather_soa_to_aos(const float* __restrict__ src, int ld_src, i
 }
 
 // ------------------------------------------------------------------------------ launchers
-static cudaError_t s1_prepare(const Scalars& sc) {
-    size_t bytes = s1_smem_bytes(sc);
-    cudaError_t e = allow_max_dynamic_smem(k_place_sample_cost, bytes);
+// Towers run instantiations without the packing's evaluation, which takes registers from theirs (descending
+// 4096 10-block towers: 412 us in the general kernel, 400 in the tower's; 64 one-block towers: 81 and 68 us).  The general
+// one keeps both goals although packings alone come to it: compiled without the tower's evaluation, the
+// packing's linear steps contract other products into FMAs, and a descent through contacts ends elsewhere.
+template <typename Kernel, typename... Args>
+static cudaError_t s1_launch(Kernel tower, Kernel any, const Scalars& sc, int n, cudaStream_t st, Args... args) {
+    if (n <= 0) return cudaSuccess;
+    const Kernel k = sc.kind == kKindPack ? any : tower;
+    const size_t bytes = s1_smem_bytes(sc);
+    cudaError_t e = allow_max_dynamic_smem(k, bytes);
     if (e != cudaSuccess) return e;
-    e = allow_max_dynamic_smem(k_place_eval, bytes);
-    if (e != cudaSuccess) return e;
-    return allow_max_dynamic_smem(k_place_descend, bytes);
+    k<<<(n + kS1Warps - 1) / kS1Warps, kS1Threads, bytes, st>>>(sc, args...);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_place_sample_cost(const Scalars& sc, DevTables t, int n, uint32_t attempt, float* x, float* cost,
                                      int* err, cudaStream_t st, const LoopCtl* ctl) {
-    if (n <= 0) return cudaSuccess;
-    cudaError_t e = s1_prepare(sc);
-    if (e != cudaSuccess) return e;
-    k_place_sample_cost<<<(n + kS1Warps - 1) / kS1Warps, kS1Threads, s1_smem_bytes(sc), st>>>(sc, t, n, attempt, x,
-                                                                                               cost, err, ctl);
-    return cudaGetLastError();
+    return s1_launch(k_place_sample_cost<true>, k_place_sample_cost<false>, sc, n, st, t, n, attempt, x, cost, err, ctl);
 }
 
 cudaError_t launch_place_eval(const Scalars& sc, DevTables t, int n, const float* x, int quad, float* cost, float* grad,
                               float* metrics, float* terms, int* err, cudaStream_t st) {
-    if (n <= 0) return cudaSuccess;
-    cudaError_t e = s1_prepare(sc);
-    if (e != cudaSuccess) return e;
-    k_place_eval<<<(n + kS1Warps - 1) / kS1Warps, kS1Threads, s1_smem_bytes(sc), st>>>(sc, t, n, x, quad, cost, grad,
-                                                                                        metrics, terms, err);
-    return cudaGetLastError();
+    return s1_launch(k_place_eval<true>, k_place_eval<false>, sc, n, st, t, n, x, quad, cost, grad, metrics, terms, err);
 }
 
 cudaError_t launch_place_descend(const Scalars& sc, DevTables t, int m, const float* x_src, int ld_src, const int* idx,
                                  float* x_dst, int k_lin, int k_quad, float* cost, int* sat, float* metrics, int* err,
                                  cudaStream_t st) {
-    if (m <= 0) return cudaSuccess;
-    cudaError_t e = s1_prepare(sc);
-    if (e != cudaSuccess) return e;
-    k_place_descend<<<(m + kS1Warps - 1) / kS1Warps, kS1Threads, s1_smem_bytes(sc), st>>>(
-        sc, t, m, x_src, ld_src, idx, x_dst, k_lin, k_quad, cost, sat, metrics, err);
-    return cudaGetLastError();
+    return s1_launch(k_place_descend<true>, k_place_descend<false>, sc, m, st, t, m, x_src, ld_src, idx, x_dst, k_lin,
+                     k_quad, cost, sat, metrics, err);
 }
 
 static int next_pow2(int v) {

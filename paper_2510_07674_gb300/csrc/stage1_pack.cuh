@@ -17,15 +17,15 @@
 // Bound by instruction issue.  The 32 spheres of a pass (four cubes) meet the cubes below whose boxes
 // they reach: one ballot per 32 cubes, in the order of the cubes, so the sums stay those of all of them.
 // The cubes' boxes are laid out once per evaluation: 32 lanes that index the constant bank by cube in
-// every pass cost more than the cull saves (4.88 -> 5.26 ms).  A handful of walls is tested without a
-// cull, which costs as much as they do.  Descending 4096 packings of 8 blocks: 4.88 -> 4.30 ms.
+// every pass cost more than the cull saves (4.88 -> 5.26 ms).  The walls' boxes (wall: centre, then half
+// extents) are laid out once per CTA.  Descending 4096 packings of 8 blocks: 4.88 -> 3.99 ms.
 #pragma once
 #include "stage1.cuh"
 
 namespace spasm {
 
-__device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const float4* __restrict__ cub, int n_cub,
-                                                     const float4* __restrict__ osph, int n_osph, const float* x,
+__device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const float4* __restrict__ cub, const float4* __restrict__ wall,
+                                                     int n_cub, const float4* __restrict__ osph, int n_osph, const float* x,
                                                      bool quad, int mode, const float* b_in, float s_coll_in,
                                                      float* g, PlaceScratch& ps, float4* gcell, float4* cube,
                                                      PlaceOut* out) {
@@ -70,8 +70,16 @@ __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const fl
         const float lz = ((m & 4) ? 0.25f : -0.25f) * u;
         const float cx = x[4 * j] + c * lx - s * ly, cy = x[4 * j + 1] + s * lx + c * ly, cz = x[4 * j + 2] + lz;
         float ax = 0.f, ay = 0.f, az = 0.f;   // dC/dc of this sphere (scaled by 2 pen in the quadratic form)
-        if (valid) {
-            for (int o = 0; o < n_cub; ++o) {
+        const SphereBox sb = warp_sphere_box(valid, cx, cy, cz, r);
+        for (int first = 0; first < n_cub; first += 32) {
+            bool near_wall = false;
+            if (first + lane < n_cub) {
+                const float4 q = wall[2 * (first + lane)], e = wall[2 * (first + lane) + 1];
+                near_wall = sb.near_box(q.x, q.y, q.z, e.x, e.y, e.z);
+            }
+            unsigned walls = __ballot_sync(0xffffffffu, near_wall);
+            for (; valid && walls; walls &= walls - 1u) {
+                const int o = first + __ffs(walls) - 1;
                 float gx, gy, gz;
                 const float pen = pen_cuboid<float>(cx, cy, cz, r, cub[4 * o], cub[4 * o + 1], cub[4 * o + 2],
                                                     cub[4 * o + 3], gx, gy, gz);
@@ -82,6 +90,8 @@ __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const fl
                     ax += sg * gx; ay += sg * gy; az += sg * gz;
                 }
             }
+        }
+        if (valid) {
             for (int o = 0; o < n_osph; ++o) {
                 float gx, gy, gz;
                 const float pen = pen_sphere<float>(cx, cy, cz, r, osph[o], gx, gy, gz);
@@ -94,7 +104,6 @@ __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const fl
             }
         }
         // cubes of the blocks below j in the skeleton order, those near the 32 spheres of this pass
-        const SphereBox sb = warp_sphere_box(valid, cx, cy, cz, r);
         unsigned long long near_cubes = 0ull;
         for (int first = 0; first < sc.n_cells; first += 32) {
             bool near_cube = false;
@@ -171,13 +180,14 @@ __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const fl
     __syncwarp();
 }
 
-// The placement cost of the problem's goal (tower or packing).
-__device__ __forceinline__ void place_eval(const Scalars& sc, const float4* __restrict__ cub, int n_cub,
-                                           const float4* __restrict__ osph, int n_osph, const float* x, bool quad,
+// The placement cost of the problem's goal (tower or packing; kTower: a tower).
+template <bool kTower>
+__device__ __forceinline__ void place_eval(const Scalars& sc, const float4* __restrict__ cub, const float4* __restrict__ wall,
+                                           int n_cub, const float4* __restrict__ osph, int n_osph, const float* x, bool quad,
                                            int mode, float* g, PlaceScratch& ps, float4* gcell, float4* cube,
                                            uint32_t* cand, PlaceOut* out) {
-    if (sc.kind == kKindPack)
-        place_eval_pack_warp(sc, cub, n_cub, osph, n_osph, x, quad, mode, nullptr, 0.f, g, ps, gcell, cube, out);
+    if (!kTower && sc.kind == kKindPack)
+        place_eval_pack_warp(sc, cub, wall, n_cub, osph, n_osph, x, quad, mode, nullptr, 0.f, g, ps, gcell, cube, out);
     else
         place_eval_warp(sc, cub, n_cub, osph, n_osph, x, quad, mode, nullptr, nullptr, 0.f, g, ps, cand, out);
 }
