@@ -481,7 +481,8 @@ def run_forms(args, rank, overrides, peak):
     """The same heterogeneous problems (1-10 blocks, 8-64 cuboids, 1024-4096 trajectory
     particles, 32 waypoints per segment) solved (a) one after another through the plain API,
     (b) as one batch (spasm_optimize_batch: one CUDA graph, one persistent trajectory
-    launch; schedule from spasm_batch_autotune on a separate copy of the problems), (c) all
+    launch; schedule from spasm_batch_autotune on a separate copy of the problems; then with
+    the launch shapes left to the library), (c) all
     submitted at once to the continuous-batching service (epochs: one batched trajectory
     attempt of every request in flight); then (d) Poisson arrivals at each rate to the
     service, latency from arrival to completion.  Problem creation and the
@@ -525,20 +526,27 @@ def run_forms(args, rank, overrides, peak):
     sched = S.spasm_batch_autotune(tune, stream=stream.cuda_stream)
     for p in tune:
         p.close()
-    torch.cuda.synchronize()
-    t0 = time.perf_counter()
-    prs = [S.Problem(wl, stream=stream.cuda_stream, **ov) for wl in wls]
-    S.spasm_optimize_batch(prs, stream=stream.cuda_stream, config=sched)
-    ok = flop = 0
-    for wl, p in zip(wls, prs):
-        r = S.spasm_result(p, allow_empty=True)
-        ok += int(r["success"].sum() > 0)
-        flop += solve_flop(wl, S.spasm_get_stats(p))
-        p.close()
-    torch.cuda.synchronize()
-    batched = form(time.perf_counter() - t0, ok, flop, schedule=sched,
-                   form="spasm_optimize_batch: stage-1 graph + stage-2 graph with one persistent trajectory launch")
-    batched["speedup_vs_plain"] = batched["solves_per_s"] / plain["solves_per_s"]
+
+    def batch(config, **extra):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        prs = [S.Problem(wl, stream=stream.cuda_stream, **ov) for wl in wls]
+        S.spasm_optimize_batch(prs, stream=stream.cuda_stream, config=config)
+        ok = flop = 0
+        for wl, p in zip(wls, prs):
+            r = S.spasm_result(p, allow_empty=True)
+            ok += int(r["success"].sum() > 0)
+            flop += solve_flop(wl, S.spasm_get_stats(p))
+            p.close()
+        torch.cuda.synchronize()
+        res = form(time.perf_counter() - t0, ok, flop, **extra)
+        res["speedup_vs_plain"] = res["solves_per_s"] / plain["solves_per_s"]
+        return res
+
+    batched = batch(sched, schedule=sched,
+                    form="spasm_optimize_batch: stage-1 graph + stage-2 graph with one persistent trajectory launch")
+    batched["library_shapes"] = batch(
+        None, form="spasm_optimize_batch without a schedule: one persistent trajectory launch per launch shape")
 
     def epoch_stats(before, after):
         e = max(after["epochs"] - before["epochs"], 1)
