@@ -24,8 +24,9 @@
 
 namespace spasm {
 
-__device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const float4* __restrict__ cub, const float4* __restrict__ wall,
-                                                     int n_cub, const float4* __restrict__ osph, int n_osph, const float* x,
+__device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const float4* __restrict__ cub,
+                                                     const float4* __restrict__ wall, int n_cub,
+                                                     const float4* __restrict__ osph, int n_osph, const float* x,
                                                      bool quad, int mode, const float* b_in, float s_coll_in,
                                                      float* g, PlaceScratch& ps, float4* gcell, float4* cube,
                                                      PlaceOut* out) {
@@ -182,8 +183,9 @@ __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const fl
 
 // The placement cost of the problem's goal (tower or packing; kTower: a tower).
 template <bool kTower>
-__device__ __forceinline__ void place_eval(const Scalars& sc, const float4* __restrict__ cub, const float4* __restrict__ wall,
-                                           int n_cub, const float4* __restrict__ osph, int n_osph, const float* x, bool quad,
+__device__ __forceinline__ void place_eval(const Scalars& sc, const float4* __restrict__ cub,
+                                           const float4* __restrict__ wall, int n_cub,
+                                           const float4* __restrict__ osph, int n_osph, const float* x, bool quad,
                                            int mode, float* g, PlaceScratch& ps, float4* gcell, float4* cube,
                                            uint32_t* cand, PlaceOut* out) {
     if (!kTower && sc.kind == kKindPack)
