@@ -1552,6 +1552,9 @@ __global__ void __launch_bounds__(kTThreads, 2) k_traj_batch(const TrajJob* __re
         }
         grp_sync<kPpc>();
         const int it = s_item[g], j = s_job[g];
+        // every thread has the item before thread 0 takes the next one: an item of the same problem that
+        // has no particle to run (a problem without a placement) meets no other barrier on its way there
+        grp_sync<kPpc>();
         if (j < 0) break;
         const TrajJob& job = jobs[j];
         if (j != cur) {
