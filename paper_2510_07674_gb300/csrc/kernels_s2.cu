@@ -1453,6 +1453,9 @@ __device__ __forceinline__ bool stage_tables_grp(void* dst0, const void* src0, u
         }
         *okw = 1u;
     }
+    // the copies write, through the async proxy, memory that the group has read and written before (the
+    // last problem's tables, boxes and state): each thread's accesses are ordered before them
+    fence_proxy_async();
     grp_sync<kPpc>();
     if (grp_tid<kPpc>() == 0) {
         mbar_expect_tx(bar, bytes0 + bytes1);
