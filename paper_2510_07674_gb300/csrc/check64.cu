@@ -17,7 +17,10 @@
 // the scene's extent), so the configuration that holds the FP64 maximum is always among those
 // repeated, and the metrics are those of the full FP64 evaluation: 85 us for the same 32 (the
 // screen 55, beside the FP64 metrics' latency, the second pass 31).
-// Joints too large for an FP32 angle, or NaN, are repeated always.
+// Configurations with a joint too large for an FP32 angle, or NaN, are repeated always, and so are
+// those that can touch a placed block whose pose FP32 does not give to the margin: its place
+// configuration has such a joint, or holds the block's x axis near the vertical, where the yaw
+// amplifies the rotation's rounding without bound.
 #include "check64.h"
 #include "stage2.cuh"
 
@@ -80,6 +83,8 @@ constexpr int kScrCfgs = 4 * kScrWarps;   // configurations per CTA of the scree
 constexpr int kChkThreads = 128, kChkWarps = kChkThreads / 32;
 constexpr float kNone = -3.4e38f;         // no obstacle within the margin
 constexpr float kMaxAngle = 8.f;          // largest joint value the FP32 evaluation takes
+constexpr float kMinLevel2 = 0.25f;       // least squared horizontal part of a placed block's x axis (unit length):
+                                          // the yaw's error is at most twice the rotation's
 
 struct ScreenWarp {
     float4 F[4][8][3];   // frames 0..7 of the warp's configurations: rows (R_i0, R_i1, R_i2, o_i)
@@ -89,6 +94,7 @@ struct ScreenShared {
     ScreenWarp warp[kScrWarps];
     float4 blk[2 * kMaxB][4];   // block cuboids: k placed, 16 + k at the initial pose
     float4 box[kMaxCub + kMaxOSph + 2 * kMaxB][2];   // boxes: environment, then the blocks
+    unsigned loose;             // bit k: FP32 does not give the pose of placed block k
 };
 
 __device__ __forceinline__ void cuboid_box(const float4* c, float4* box) {
@@ -266,16 +272,20 @@ __global__ void __launch_bounds__(kScrThreads) k_check_screen(const __grid_const
         }
         fk_lanes<float>(sc, sn, cs, R, o);
     };
+    if (tid == 0) sh.loose = 0u;
+    __syncthreads();
     // the blocks' cuboids and every obstacle's box
     if (!p2p) {
         for (int g = w; 4 * g < B; g += kScrWarps) {
             const int b = min(4 * g + (lane >> 3), B - 1);
             float R[9], o[3], Rt[9], pt[3], Rb[9], pb[3];
-            bool x, y;
-            kinematics(t_place(S, b), R, o, x, y);
+            bool outside, large;
+            kinematics(t_place(S, b), R, o, outside, large);
+            const unsigned joints = __ballot_sync(0xffffffffu, large) >> (lane & ~7) & 0xffu;
             if (k == 7) {
                 tool_frame<float>(sc, R, o, Rt, pt);
                 held_block<float>(sc, b, Rt, pt, Rb, pb);
+                if (joints || !(Rb[0] * Rb[0] + Rb[3] * Rb[3] >= kMinLevel2)) atomicOr(&sh.loose, 1u << b);
                 block_cuboid(pb[0], pb[1], pb[2], atan2f(Rb[3], Rb[0]), sc.half[b], sh.blk[b]);
                 cuboid_box(sh.blk[b], sh.box[n_env + b]);
             }
@@ -318,6 +328,7 @@ __global__ void __launch_bounds__(kScrThreads) k_check_screen(const __grid_const
         }
         __syncwarp();
     }
+    const unsigned loose = sh.loose;
     float top = kNone;
 #pragma unroll 1
     for (int ci = 0; ci < nc; ++ci) {
@@ -384,7 +395,7 @@ __global__ void __launch_bounds__(kScrThreads) k_check_screen(const __grid_const
             }
         }
         v = warp_fmax(v);
-        const bool force = (forced >> (8 * ci)) & 0xffu;
+        const bool force = ((forced >> (8 * ci)) & 0xffu) || (loose & ((1u << b) - 1u));   // placed blocks k < b
         if (lane == 0) val[(size_t)r * C + t] = force ? INFINITY : v;
         if (!force) top = fmaxf(top, v);
     }

@@ -1,0 +1,73 @@
+"""The FP64 check where a placed block's pose cannot be had in FP32: its place configuration has
+joints too large for an FP32 angle (on a robot with joint offsets, where the sum of the two rounds), or
+holds the block's x axis vertical, so that its yaw hangs on the last bits.  The blocks' later
+configurations reach into it; the metrics are the oracle's (1e-9 relative, as for every check)."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2510_07674_gb300 import scenes
+from test_gpu_check64 import _compare, _float_limits, _gpu_check
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+B, W, N_TRAJ = 3, 8, 24
+
+
+def _workload(offsets=0.0):
+    wl = scenes.make_problem("tower4", seed=4, B=B, O=0, W=W, N=64, M=16, P=4, Q=4, ik_mode=0)
+    wl.scene.cuboid = np.zeros((0, 15))   # nothing but the blocks
+    wl.scene.half = np.array([[0.04, 0.015, 0.025]] * B)
+    wl.robot.dh[:, 3] = offsets
+    return wl
+
+
+def _upright(orc, rng):
+    """A configuration whose tool x axis is vertical up to 2e-6: Newton steps on its horizontal part."""
+    angle = rng.uniform(-np.pi, np.pi)
+    target = 2e-6 * np.array([np.cos(angle), np.sin(angle)])
+
+    def res(q):
+        return orc.fk(q)[1][:2, 0] - target
+    q = rng.uniform(-1.0, 1.0, 7) + np.array([0, 0, 0, -1.5, 0, 1.0, 0])
+    for _ in range(60):
+        r = res(q)
+        J = np.stack([(res(q + 1e-6 * e) - r) / 1e-6 for e in np.eye(7)], 1)
+        q = q - np.clip(np.linalg.pinv(J, rcond=1e-6) @ r, -0.3, 0.3)
+    assert np.abs(res(q)).max() < 1e-9
+    return q
+
+
+def _trajectories(kind, wl, orc):
+    rng = np.random.default_rng(8)
+    S = W - 1
+    C = 2 * B * S + 1
+    q = np.repeat(wl.robot.q_home[None, None], N_TRAJ, 0).repeat(C, 1)
+    q += rng.uniform(-0.3, 0.3, q.shape)
+    for p in range(N_TRAJ):
+        t = 2 * S                                              # block 0's place configuration
+        if kind == "large":
+            far = rng.uniform(-1.0, 1.0, 7) + 2 * np.pi * rng.integers(20000, 40000, 7)
+            q[p, t] = far.astype(np.float32)
+            near = np.mod(q[p, t] + np.pi, 2 * np.pi) - np.pi   # the same angles
+        else:
+            q[p, t] = near = _upright(orc, rng)
+        spread = 0.08 if kind == "large" else 0.01
+        q[p, t + 1:] = near + rng.uniform(-spread, spread, (C - t - 1, 7))
+    return q
+
+
+@pytest.mark.parametrize("kind", ["large", "vertical"])
+def test_placed_blocks_that_fp32_cannot_place(kind):
+    from paper_2510_07674_gb300 import spasm as S
+    wl = _workload(np.array([0.3, -0.7, 1.1, -0.2, 0.9, -1.3, 0.5]) if kind == "large" else 0.0)
+    orc = O.Oracle(_float_limits(wl))
+    q = _trajectories(kind, wl, orc)
+    pr = S.Problem(wl)
+    try:
+        q32, m, ok = _gpu_check(pr, q)
+        _compare(orc, q32, m, ok)
+        assert (m[:, 0] > 1e-3).sum() >= 12   # the arm is in the placed block
+    finally:
+        pr.close()
