@@ -363,7 +363,10 @@ static spasm_status create_problem_impl(const spasm_robot* robot, const spasm_ob
         }
         q.grasp_off = goal->grasp_off; q.eps = prm->eps; q.eps_start = prm->eps_start;
         // the FP32 screen's margin: 2e-5 (335 rounding steps) of the scene's extent, the arm's length with
-        // its largest sphere or held block and the farthest obstacle point from the origin
+        // its largest sphere or held block and the farthest obstacle point from the origin.  Angles add
+        // their own rounding, 2^-23 of their size: a joint's offset (the offset and its sum with the joint,
+        // half of that each) times the arm's length, a block's initial yaw times the block's size; 2.5e-7
+        // is twice that
         auto norm3 = [](const double* v) { return std::sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]); };
         double arm = 0.0, far = 0.0, held = 0.0;
         for (int k = 0; k < 7; ++k) arm += std::fabs(q.a[k]) + std::fabs(q.d[k]);
@@ -375,7 +378,11 @@ static spasm_status create_problem_impl(const spasm_robot* robot, const spasm_ob
         }
         for (int o = 0; o < sc.n_cub; ++o) far = std::fmax(far, norm3(obs->cuboid + 15 * o) + norm3(obs->cuboid + 15 * o + 12));
         for (int o = 0; o < sc.n_osph; ++o) far = std::fmax(far, norm3(obs->sphere + 4 * o) + std::fabs(obs->sphere[4 * o + 3]));
-        q.margin = (float)(2e-5 * (arm + norm3(q.ee_p) + tip + held + far));
+        double offsets = 0.0, turned = 0.0;
+        for (int k = 0; k < 7; ++k) offsets += std::fabs(q.th0[k]);
+        for (int i = 0; i < B; ++i) turned = std::fmax(turned, std::fabs(q.init[i][3]) * norm3(q.half[i]));
+        const double reach = arm + norm3(q.ee_p) + tip + held;
+        q.margin = (float)(2e-5 * (reach + far) + 2.5e-7 * (offsets * reach + turned));
     }
     pr->host_osph.assign(obs->sphere, obs->sphere + 4 * (size_t)sc.n_osph);
 

@@ -14,9 +14,9 @@
 //                   margin of the solution's largest (and above minus the margin: below, nothing
 //                   is penetrated), a warp per configuration; usually one or two of 620.
 // The margin bounds the FP32 evaluation's error (Scalars64::margin, some hundred rounding steps of
-// the scene's extent), so the configuration that holds the FP64 maximum is always among those
-// repeated, and the metrics are those of the full FP64 evaluation: 85 us for the same 32 (the
-// screen 55, beside the FP64 metrics' latency, the second pass 31).
+// the scene's extent, more where the joints have offsets), so the configuration that holds the FP64
+// maximum is always among those repeated, and the metrics are those of the full FP64 evaluation:
+// 85 us for the same 32 (the screen 55, beside the FP64 metrics' latency, the second pass 31).
 // Configurations with a joint too large for an FP32 angle, or NaN, are repeated always, and so are
 // those that can touch a placed block whose pose FP32 does not give to the margin: its place
 // configuration has such a joint, or holds the block's x axis near the vertical, where the yaw

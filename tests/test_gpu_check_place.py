@@ -1,7 +1,8 @@
 """The FP64 check where a placed block's pose cannot be had in FP32: its place configuration has
 joints too large for an FP32 angle (on a robot with joint offsets, where the sum of the two rounds), or
 holds the block's x axis vertical, so that its yaw hangs on the last bits.  The blocks' later
-configurations reach into it; the metrics are the oracle's (1e-9 relative, as for every check)."""
+configurations reach into it; the metrics are the oracle's (1e-9 relative, as for every check).
+And robots whose joint offsets, blocks whose yaws, are of many turns."""
 import numpy as np
 import pytest
 
@@ -69,5 +70,27 @@ def test_placed_blocks_that_fp32_cannot_place(kind):
         q32, m, ok = _gpu_check(pr, q)
         _compare(orc, q32, m, ok)
         assert (m[:, 0] > 1e-3).sum() >= 12   # the arm is in the placed block
+    finally:
+        pr.close()
+
+
+@pytest.mark.parametrize("offset", [50.0, 10000.0])
+def test_joint_offsets_and_yaws_that_round_in_fp32(offset):
+    """Joint offsets and initial yaws of many turns: their FP32 rounding moves every sphere and every
+    block at its initial pose by more than the arithmetic's own rounding does."""
+    from paper_2510_07674_gb300 import spasm as S
+    turns = 2 * np.pi * np.round(offset / (2 * np.pi))
+    wl = _workload(turns + np.array([0.3, -0.7, 1.1, -0.2, 0.9, -1.3, 0.5]))
+    wl.scene.init[:, 3] += turns
+    orc = O.Oracle(_float_limits(wl))
+    rng = np.random.default_rng(3)
+    C = 2 * B * (W - 1) + 1
+    q = rng.uniform(-1.0, 1.0, (N_TRAJ, 1, 7)) + rng.uniform(-0.2, 0.2, (N_TRAJ, C, 7))
+    q[:, 2 * (W - 1) + 1:] = q[:, [2 * (W - 1)]] + rng.uniform(-0.08, 0.08, (N_TRAJ, C - 2 * (W - 1) - 1, 7))
+    pr = S.Problem(wl)
+    try:
+        q32, m, ok = _gpu_check(pr, q)
+        _compare(orc, q32, m, ok)
+        assert (m[:, 0] > 1e-3).sum() >= 12
     finally:
         pr.close()
