@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(kScrThreads) k_check_screen(const __grid_const
         outside = large = false;
         if (k > 0) {
             const float v = qr[t * 8 + k - 1];
-            outside = v < sc.qlo[k - 1] || v > sc.qhi[k - 1];
+            outside = v < sc.qlo[k - 1] || v > sc.qhi[k - 1] || !isfinite(v);   // nothing else refuses a NaN
             large = !(fabsf(v) <= kMaxAngle);
             sincosf(sc.th0[k - 1] + v, &sn, &cs);
         }
