@@ -18,6 +18,11 @@
  *   - Work is enqueued on the problem's CUDA stream (set at creation) and is
  *     asynchronous unless the function says it synchronises.
  *   - Calls on one problem handle are not thread-safe; distinct handles are.
+ *   - The kernel-level calls can be captured into CUDA graphs (on the problem's stream).
+ *     Captured, they share nothing that they write with other calls on the handle but its
+ *     error word, so that graphs of them may be replayed side by side; spasm_traj_check,
+ *     whose accumulators are the handle's, and spasm_place_select_static, whose array is the
+ *     device's, may not.
  *   - Device errors (a bounded wait that gave up, a size outside the compiled limits)
  *     are recorded in a per-problem error word and reported as SPASM_ERR_DEVICE by the
  *     next synchronising call.

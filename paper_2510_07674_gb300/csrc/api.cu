@@ -636,6 +636,16 @@ extern "C" spasm_status spasm_lift(spasm_problem_t pr, int n, const float* place
     return SPASM_OK;
 }
 
+// The handle's scratch for a trajectory launch on its stream, where launches follow one another; none
+// while that stream is being captured, as graphs may be replayed on any streams, side by side.
+static void take_scratch(spasm_problem* pr, TrajIO& io) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(pr->stream, &cs) != cudaSuccess) cudaGetLastError();   // the launch will say it
+    if (cs != cudaStreamCaptureStatusNone) return;
+    io.rows = pr->d_rows;
+    io.work = pr->d_work;
+}
+
 extern "C" spasm_status spasm_traj_eval(spasm_problem_t pr, int n, const float* q, const float* lam, const float* mu,
                                         float* L, float* grad, float* groups, float* h) {
     if (!pr || n < 0 || (n > 0 && !q)) return fail(SPASM_ERR_INVALID, "bad arguments");
@@ -644,7 +654,7 @@ extern "C" spasm_status spasm_traj_eval(spasm_problem_t pr, int n, const float* 
     io.lam = const_cast<float*>(lam);
     io.mu = const_cast<float*>(mu);
     io.L = L; io.grad = grad; io.groups = groups; io.h = h;
-    io.rows = pr->d_rows; io.work = pr->d_work;
+    take_scratch(pr, io);
     SPASM_CUDA(launch_traj(pr->sc, pr->tab, n, kTrajModeEval, io, pr->d_err, pr->stream));
     return SPASM_OK;
 }
@@ -656,7 +666,7 @@ extern "C" spasm_status spasm_traj_descend(spasm_problem_t pr, int n, float* q, 
     TrajIO io{};
     io.q = q; io.lam = lam; io.mu = mu; io.metrics = metrics; io.sat = sat;
     io.k_steps = k_steps; io.init_multipliers = init_multipliers;
-    io.rows = pr->d_rows; io.work = pr->d_work;
+    take_scratch(pr, io);
     SPASM_CUDA(launch_traj(pr->sc, pr->tab, n, kTrajModeDescend, io, pr->d_err, pr->stream));
     return SPASM_OK;
 }

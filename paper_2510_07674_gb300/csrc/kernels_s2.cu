@@ -166,6 +166,9 @@ static size_t t_region(int C, int B, int ppc) {
            ~(size_t)127;
 }
 
+// The collision gradient rows of one particle, as the tail of its region in a launch without scratch.
+__host__ __device__ inline size_t t_rows_bytes(int C) { return ((size_t)C * 16 * sizeof(float) + 127) & ~(size_t)127; }
+
 size_t traj_cta_smem_bytes(const TrajScalars& sc, int ppc, bool batched) {
     const size_t env = t_env_bytes(sc.n_cub, sc.n_osph);
     return (batched ? ppc : 1) * env + ppc * t_region(sc.C, sc.B, ppc);
@@ -1477,8 +1480,10 @@ __device__ __forceinline__ bool stage_tables_grp(void* dst0, const void* src0, u
 // Persistent grid over n particles, kPpc groups per CTA: a group starts with particle = its
 // index and takes the next one from the work counter when it is done, so that particles of
 // uneven length keep every group busy to the end; the group that finishes last leaves the
-// counters at zero for the next launch.  The problem's tables and constants are staged once
-// per group.  (kP2P: the point-to-point instantiation; kTile: the sphere tiling.)
+// counters at zero for the next launch.  The problem's tables are staged once per CTA, its
+// constants once per group.  (kP2P: the point-to-point instantiation; kTile: the sphere tiling.)
+// A launch without scratch (io.rows and io.work null) has a group per particle and its gradient
+// rows in shared memory, so that nothing of it is shared with any other launch.
 template <bool kP2P, int kTile, int kPpc>
 __global__ void __launch_bounds__(kTThreads, 2) k_traj(const __grid_constant__ Scalars sc, DevTables tab, int n, int mode,
                                                        TrajIO io, int* err, int region_bytes) {
@@ -1496,15 +1501,17 @@ __global__ void __launch_bounds__(kTThreads, 2) k_traj(const __grid_constant__ S
         group_setup<kPpc>(sc, sh);
         __syncthreads();
         const LaneSpheres ls = lane_spheres<kTile>(sc);
-        float* rows = io.rows + (size_t)slot * sc.C * 16;
+        float* rows = io.rows ? io.rows + (size_t)slot * sc.C * 16
+                              : reinterpret_cast<float*>(region + region_bytes - t_rows_bytes(sc.C));
         for (int p = slot; p < n;) {
             traj_particle<kP2P, kTile, kPpc>(sc, ls, p, mode, io, rows, smem_all, region);
+            if (!io.work) break;
             if (grp_tid<kPpc>() == 0) sh.particle = groups + atomicAdd(&io.work->next, 1);
             grp_sync<kPpc>();   // also: the outputs were read from the region before the next particle fills it
             p = sh.particle;
         }
     }
-    if (grp_tid<kPpc>() == 0) {
+    if (io.work && grp_tid<kPpc>() == 0) {
         __threadfence();
         if (atomicAdd(&io.work->done, 1) == groups - 1) {
             __threadfence();
@@ -1684,22 +1691,27 @@ int traj_ctas_per_sm(const TrajScalars& sc) {
 template <bool kP2P, int kTile, int kPpc>
 static cudaError_t traj_kernel(const Scalars& sc, DevTables t, int n, int mode, const TrajIO& io, int* err,
                                cudaStream_t st) {
-    const size_t dyn = traj_cta_smem_bytes(sc, kPpc, false);
+    const size_t region = t_region(sc.C, sc.B, kPpc) + (io.rows ? 0 : t_rows_bytes(sc.C));
+    const size_t dyn = t_env_bytes(sc.n_cub, sc.n_osph) + kPpc * region;
     int sms = 0;
     size_t half = 0;
     cudaError_t e = sm_limits(&sms, &half);
     if (e == cudaSuccess) e = allow_max_dynamic_smem(k_traj<kP2P, kTile, kPpc>, dyn);
     if (e != cudaSuccess) return e;
     const int resident = std::min(sms * (dyn <= half ? 2 : 1), traj_slots(sc.B, sc.C, sc.n_cub, sc.n_osph) / kPpc);
-    const int grid = std::min((n + kPpc - 1) / kPpc, resident);
-    k_traj<kP2P, kTile, kPpc><<<grid, kTThreads, dyn, st>>>(sc, t, n, mode, io, err, (int)t_region(sc.C, sc.B, kPpc));
+    const int all = (n + kPpc - 1) / kPpc, grid = io.rows ? std::min(all, resident) : all;
+    k_traj<kP2P, kTile, kPpc><<<grid, kTThreads, dyn, st>>>(sc, t, n, mode, io, err, (int)region);
     return cudaGetLastError();
 }
 
 template <bool kP2P>
 static cudaError_t traj_dispatch(const Scalars& sc, DevTables t, int n, int mode, const TrajIO& io, int* err,
                                  cudaStream_t st) {
-    const int ppc = traj_ppc(sc, n);
+    int ppc = traj_ppc(sc, n);
+    if (!io.rows) {   // with their rows in shared memory fewer particles share a CTA
+        const size_t env = t_env_bytes(sc.n_cub, sc.n_osph), rows = t_rows_bytes(sc.C);
+        while (ppc > 1 && env + ppc * (t_region(sc.C, sc.B, ppc) + rows) > kHalfSmem) ppc /= 2;
+    }
     if (ppc == 4) return traj_kernel<kP2P, 0, 4>(sc, t, n, mode, io, err, st);
     if (ppc == 2)
         return sc.sphere_tiling ? traj_kernel<kP2P, 1, 2>(sc, t, n, mode, io, err, st)

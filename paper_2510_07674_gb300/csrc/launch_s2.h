@@ -28,9 +28,11 @@ struct TrajIO {
     int init_multipliers;   // descent starts from lambda = 0, mu = mu0
     const int* active;  // optional device word: when it holds 0 or less the launch does nothing (the
                         // trajectory stage of a problem whose stage 1 found no placement)
-    float* rows;        // [traj_slots][C][16] scratch (required): the collision gradient rows of the
-                        // particle each resident group works on
-    TrajWork* work;   // the launch's work counters (required by launch_traj), zero between launches
+    // Scratch that no other launch in flight may have: the collision gradient rows of the particle each
+    // resident group works on, [traj_slots][C][16], and launch_traj's work counters, zero between
+    // launches.  launch_traj takes neither as well (both null): the rows then lie in shared memory.
+    float* rows;
+    TrajWork* work;
 };
 // Particle groups resident at once: two CTAs of two groups on each of 152 SMs, or of four where
 // the problem is small enough (traj_slots); a launch on a part with more SMs keeps to as many.
