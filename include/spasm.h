@@ -144,9 +144,12 @@ typedef struct {
  * C <= 1024, N <= 32768, M <= 8192, P <= M, Q >= 1.  Synchronises once. */
 spasm_status spasm_create_problem(const spasm_robot* robot, const spasm_obstacles* obstacles, const spasm_goal* goal,
                                   const spasm_params* params, void* cuda_stream, spasm_problem_t* out);
-/* Device memory, in bytes, that spasm_create_problem would allocate for this problem (the
- * same buffer list, each rounded up to the pool's 512-byte granule); robot arrays do not
- * matter.  The solver service admits requests against its budget with this figure. */
+/* Device memory, in bytes, of a problem's own buffers, as spasm_create_problem allocates them
+ * (the same buffer list, each rounded up to the pool's 512-byte granule); robot arrays do not
+ * matter.  The solver service admits requests against its budget with this figure.  Not in
+ * it: the scratch of the trajectory launches, 64 C bytes for each of the 608 particle groups
+ * that can run at once (1216 for small problems) whatever Q is, which spasm_create_problem
+ * and spasm_create_p2p allocate besides and the service has once for all its requests. */
 spasm_status spasm_problem_bytes(const spasm_obstacles* obstacles, const spasm_goal* goal, const spasm_params* params,
                                  long long* bytes);
 /* A packing problem (the appendix's Tetris problem) for stage 1 (spasm_place, the
@@ -445,7 +448,8 @@ spasm_status spasm_batch_autotune(spasm_problem_t* problems, int n, void* cuda_s
  * Requests are whole problems (copied at submission).  One scheduler thread runs the device
  * work in epochs, each one trajectory attempt of every request in flight: queued requests are
  * admitted in arrival order while fewer than max_inflight are in flight and their device
- * memory (spasm_problem_bytes) fits budget_bytes (a request larger than the whole budget is
+ * memory (spasm_problem_bytes) fits budget_bytes, beside which the service holds the scratch of
+ * its trajectory launches, at most 2 x 38 MB (a request larger than the whole budget is
  * admitted when nothing else is in flight), created on the scheduler's stream of the device
  * current at creation, and their stage 1 runs (with its device-side attempt loop); then one
  * persistent launch of the trajectory kernel per launch shape (one or two) runs the descent of the

@@ -102,7 +102,8 @@ static cudaError_t reset_loops(spasm_problem* pr) {
 extern "C" const char* spasm_last_error(void) { return g_last_error.c_str(); }
 
 // Every device buffer of a problem with its element count, in allocation order: the one list
-// that spasm_create_problem allocates and spasm_problem_bytes adds up.
+// that spasm_create_problem allocates and spasm_problem_bytes adds up.  The trajectory launches'
+// gradient rows are not in it: a launch needs them, not a problem (create_problem_impl).
 template <typename F>
 static void for_each_buffer(spasm_problem* pr, int B, int C, int n_cub, int n_osph, const spasm_params* prm, F&& f) {
     const size_t N = prm->N, M = prm->M, P = prm->P, Q = prm->Q, NR = 9 * (size_t)B + 3;
@@ -137,7 +138,6 @@ static void for_each_buffer(spasm_problem* pr, int B, int C, int n_cub, int n_os
     f(pr->d_sc, 1);
     f(pr->d_chkacc, P);
     f(pr->d_ctl, 1);
-    f(pr->d_rows, (size_t)traj_slots(B, C, n_cub, n_osph) * C * 16);
     f(pr->d_work, 1);
     f(pr->d_chkval, P * (size_t)C);
 }
@@ -176,8 +176,11 @@ static bool franka_layout(const double* dh) {
     return std::hypot(a3 * a4 + d2 * d4, d2 * a4 - a3 * d4) > 0.0;
 }
 
+// own_rows: the problem's trajectory launches have their gradient rows in memory of its own (24 MB for
+// the 10-block tower, whatever Q is); otherwise they come with the batched launch, or lie in shared memory.
 static spasm_status create_problem_impl(const spasm_robot* robot, const spasm_obstacles* obs, const spasm_goal* goal,
-                                        const spasm_params* prm, void* cuda_stream, spasm_problem_t* out) {
+                                        const spasm_params* prm, void* cuda_stream, spasm_problem_t* out,
+                                        bool own_rows = true) {
     Range range("spasm create problem");
     if (!robot || !obs || !goal || !prm || !out) return fail(SPASM_ERR_INVALID, "null argument");
     *out = nullptr;
@@ -390,6 +393,8 @@ static spasm_status create_problem_impl(const spasm_robot* robot, const spasm_ob
     for_each_buffer(pr, B, C, sc.n_cub, sc.n_osph, prm, [&](auto*& ptr, size_t count) {
         if (st == SPASM_OK) st = dalloc(&ptr, count, pr->stream);
     });
+    if (st == SPASM_OK && own_rows)
+        st = dalloc(&pr->d_rows, (size_t)traj_slots(B, C, sc.n_cub, sc.n_osph) * C * 16, pr->stream);
     for (auto& ev : pr->ev)
         if (st == SPASM_OK && cudaEventCreate(&ev) != cudaSuccess) st = fail(SPASM_ERR_CUDA, "cudaEventCreate failed");
     // streams the attempt-loop graphs are captured on (the problem's own stream may be the
@@ -454,6 +459,13 @@ extern "C" spasm_status spasm_create_problem(const spasm_robot* robot, const spa
     return finish_create(pr, out);
 }
 
+spasm_status spasm::create_served_problem(const spasm_robot* robot, const spasm_obstacles* obs, const spasm_goal* goal,
+                                          const spasm_params* prm, cudaStream_t stream, spasm_problem_t* out) {
+    spasm_problem_t pr = nullptr;
+    SPASM_TRY(create_problem_impl(robot, obs, goal, prm, stream, &pr, false));
+    return finish_create(pr, out);
+}
+
 extern "C" spasm_status spasm_create_packing(const spasm_robot* robot, const spasm_packing* pk,
                                              const spasm_params* prm, void* cuda_stream, spasm_problem_t* out) {
     if (!pk || !out) return fail(SPASM_ERR_INVALID, "null argument");
@@ -488,7 +500,7 @@ extern "C" spasm_status spasm_create_packing(const spasm_robot* robot, const spa
     spasm_obstacles obs{4, walls.data(), 0, nullptr};
     spasm_goal goal{B, half.data(), init.data(), box, zs - 0.5 * u, 0.0};
     spasm_problem_t pr = nullptr;
-    SPASM_TRY(create_problem_impl(robot, &obs, &goal, prm, cuda_stream, &pr));
+    SPASM_TRY(create_problem_impl(robot, &obs, &goal, prm, cuda_stream, &pr, false));   // no stage 2
     Scalars& sc = pr->sc;
     sc.kind = kKindPack;
     sc.n_cells = total;
@@ -636,12 +648,13 @@ extern "C" spasm_status spasm_lift(spasm_problem_t pr, int n, const float* place
     return SPASM_OK;
 }
 
-// The handle's scratch for a trajectory launch on its stream, where launches follow one another; none
-// while that stream is being captured, as graphs may be replayed on any streams, side by side.
+// The handle's scratch, where it has any, for a trajectory launch on its stream, where launches follow
+// one another; none while that stream is being captured, as graphs may be replayed on any streams, side
+// by side.
 static void take_scratch(spasm_problem* pr, TrajIO& io) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(pr->stream, &cs) != cudaSuccess) cudaGetLastError();   // the launch will say it
-    if (cs != cudaStreamCaptureStatusNone) return;
+    if (cs != cudaStreamCaptureStatusNone || !pr->d_rows) return;
     io.rows = pr->d_rows;
     io.work = pr->d_work;
 }

@@ -143,7 +143,8 @@ JobList make_jobs(spasm_problem_t* prs, const std::vector<int>& live, int per_fe
             j.io.tests = pr->d_tests;
             j.io.active = &pr->d_ctl->n_place;
         }
-        j.io.rows = pr->d_rows;
+        j.io.rows = pr->d_rows;   // null: prepare_batch's
+        j.io.row_stride = pr->sc.C * 16;
         j.io.k_steps = k_steps;
         j.io.init_multipliers = init_multipliers ? 1 : 0;
         j.err = pr->d_err;
@@ -213,10 +214,16 @@ spasm::BatchLaunch::~BatchLaunch() {
 }
 
 spasm_status spasm::prepare_batch(spasm_problem_t* prs, const std::vector<int>& order, const spasm_batch_config& cfg,
-                                  cudaStream_t s, BatchLaunch& bl) {
+                                  cudaStream_t s, BatchLaunch& bl, BatchRows& rows) {
     JobList L = make_jobs(prs, order, cfg.per_fetch, kTrajModeDescend, 0, true, cfg.particles_per_cta);
     for (size_t k = 0; k < order.size(); ++k) L.jobs[k].io.k_steps = prs[order[k]]->sc.K_traj;
     SPASM_TRY(batch_grid(cfg, L, &bl.grid));
+    int stride = 0;   // of the shared rows: that of the largest problem without its own
+    for (const TrajJob& j : L.jobs)
+        if (!j.io.rows) stride = std::max(stride, j.io.row_stride);
+    if (stride) SPASM_TRY(rows.reserve((size_t)bl.grid * L.ppc * stride, s));
+    for (TrajJob& j : L.jobs)
+        if (!j.io.rows) { j.io.rows = rows.p; j.io.row_stride = stride; }
     bl.host = std::move(L.jobs);
     bl.n_items = L.n_items;
     bl.cta_bytes = L.cta_bytes;
@@ -237,6 +244,21 @@ spasm_status spasm::enqueue_batch(const BatchLaunch& bl, cudaStream_t s) {
     return SPASM_OK;
 }
 
+spasm::BatchRows::~BatchRows() {
+    if (p) cudaFreeAsync(p, s);
+}
+
+spasm_status spasm::BatchRows::reserve(size_t n, cudaStream_t st) {
+    if (n <= floats) return SPASM_OK;
+    if (p) SPASM_CUDA(cudaFreeAsync(p, s));
+    p = nullptr;
+    floats = 0;
+    s = st;
+    SPASM_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&p), n * sizeof(float), st));
+    floats = n;
+    return SPASM_OK;
+}
+
 spasm::BatchSet::~BatchSet() {
     if (fork) cudaEventDestroy(fork);
     if (join) cudaEventDestroy(join);
@@ -244,8 +266,8 @@ spasm::BatchSet::~BatchSet() {
 }
 
 spasm_status spasm::prepare_batches(spasm_problem_t* prs, const std::vector<int>& order, const spasm_batch_config& cfg,
-                                    cudaStream_t s, BatchSet& set) {
-    if (cfg.particles_per_cta) return prepare_batch(prs, order, cfg, s, set.launch[0]);
+                                    cudaStream_t s, BatchSet& set, BatchRows rows[2]) {
+    if (cfg.particles_per_cta) return prepare_batch(prs, order, cfg, s, set.launch[0], rows[0]);
     std::vector<int> by[2];   // one and two particles per CTA
     long long particles = 0;
     for (int i : order) particles += prs[i]->sc.Q;
@@ -259,7 +281,8 @@ spasm_status spasm::prepare_batches(spasm_problem_t* prs, const std::vector<int>
         if (by[k].empty()) continue;
         spasm_batch_config c = cfg;
         c.particles_per_cta = k + 1;
-        SPASM_TRY(prepare_batch(prs, by[k], c, s, set.launch[n++]));
+        SPASM_TRY(prepare_batch(prs, by[k], c, s, set.launch[n], rows[n]));
+        ++n;
     }
     if (n == 2) {
         SPASM_CUDA(cudaStreamCreateWithFlags(&set.side, cudaStreamNonBlocking));
@@ -314,8 +337,9 @@ extern "C" spasm_status spasm_optimize_batch(spasm_problem_t* prs, int n, void* 
         all[i] = i;
     }
     const std::vector<int> order = job_order(prs, all, cfg.order);
+    BatchRows rows[2];
     BatchSet bl;
-    SPASM_TRY(prepare_batches(prs, order, cfg, s, bl));
+    SPASM_TRY(prepare_batches(prs, order, cfg, s, bl, rows));
     // one graph: stage 1 of the problems not yet placed, the first lift of every problem, one
     // persistent trajectory launch over all particles, then each problem's selection, re-lift
     // loop and FP64 check; problems whose stage 1 kept nothing skip stage 2 on the device

@@ -198,7 +198,7 @@ TrajIO descent_io(spasm_problem* pr) {
     io.k_steps = pr->sc.K_traj; io.init_multipliers = 1;
     io.tests = pr->d_tests;
     io.active = &pr->d_ctl->n_place;
-    io.rows = pr->d_rows; io.work = pr->d_work;
+    if (pr->d_rows) { io.rows = pr->d_rows; io.work = pr->d_work; }
     return io;
 }
 

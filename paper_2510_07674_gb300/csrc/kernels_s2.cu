@@ -1586,7 +1586,7 @@ __global__ void __launch_bounds__(kTThreads, 2) k_traj_batch(const TrajJob* __re
             cur = j;
         }
         const LaneSpheres ls = lane_spheres<kTile>(*job.sc);
-        float* rows = io_s.rows + (size_t)(blockIdx.x * kPpc + g) * sc_s.C * 16;
+        float* rows = io_s.rows + (size_t)(blockIdx.x * kPpc + g) * io_s.row_stride;
         const int p0 = (it - job.first) * per_fetch;
         // a problem whose stage 1 found no placement has nothing to optimise
         const int p1 = (io_s.active && *io_s.active <= 0) ? p0 : min(p0 + per_fetch, job.n);

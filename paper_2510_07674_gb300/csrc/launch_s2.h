@@ -33,6 +33,7 @@ struct TrajIO {
     // launches.  launch_traj takes neither as well (both null): the rows then lie in shared memory.
     float* rows;
     TrajWork* work;
+    int row_stride;   // batched launches: floats from one group's rows to the next one's
 };
 // Particle groups resident at once: two CTAs of two groups on each of 152 SMs, or of four where
 // the problem is small enough (traj_slots); a launch on a part with more SMs keeps to as many.

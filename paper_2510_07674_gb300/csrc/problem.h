@@ -49,7 +49,8 @@ struct spasm_problem {
     int *d_tsat = nullptr, *d_tnsat = nullptr, *d_tbest = nullptr;
     float *d_rq = nullptr, *d_rcost = nullptr;   // returned solutions
     int* d_rsucc = nullptr;
-    float* d_rows = nullptr;             // the trajectory kernel's gradient rows (traj_slots x C x 16)
+    float* d_rows = nullptr;             // the trajectory kernel's gradient rows (traj_slots x C x 16), or null:
+                                         // a packing, a problem of the service
     spasm::TrajWork* d_work = nullptr;   // and work counters
     unsigned long long* d_tests = nullptr;   // [tests run, configurations culled] by the trajectory kernel
     bool optimized = false;
@@ -104,6 +105,9 @@ inline spasm_status rec(spasm_problem* pr, int i) {
     return SPASM_OK;
 }
 
+// spasm_create_problem for the service, which runs stage 2 in batched launches only: without gradient rows.
+spasm_status create_served_problem(const spasm_robot* robot, const spasm_obstacles* obs, const spasm_goal* goal,
+                                   const spasm_params* prm, cudaStream_t stream, spasm_problem_t* out);
 // Makes the host wait for the problem's stream (counted in stats.host_waits).
 spasm_status host_wait(spasm_problem* pr);
 // Reads the problem's device error word (synchronises its stream).
@@ -133,6 +137,19 @@ spasm_status enqueue_traj_epoch_end(spasm_problem* pr, cudaStream_t s);
 // A persistent launch of the trajectory kernel in descent mode over the particles of several
 // problems (batch.cu): the work list lives on the device until this object is destroyed,
 // which must come after the launch has finished.
+// Gradient rows of a batched launch whose problems have none of their own; kept from one launch to the
+// next where it outlives them (the service).
+struct BatchRows {
+    float* p = nullptr;
+    size_t floats = 0;
+    cudaStream_t s = nullptr;
+    BatchRows() = default;
+    BatchRows(const BatchRows&) = delete;
+    BatchRows& operator=(const BatchRows&) = delete;
+    ~BatchRows();
+    // At least n floats; launches that used the last ones must have finished, or run before on st.
+    spasm_status reserve(size_t n, cudaStream_t st);
+};
 struct BatchLaunch {
     std::vector<TrajJob> host;   // source of the asynchronous upload
     TrajJob* jobs = nullptr;
@@ -148,7 +165,7 @@ struct BatchLaunch {
 // Builds and uploads (on s, asynchronously) the work list of problems prs[order[k]], each with
 // its own K_traj steps and its placement count as the gate.
 spasm_status prepare_batch(spasm_problem_t* prs, const std::vector<int>& order, const spasm_batch_config& cfg,
-                           cudaStream_t s, BatchLaunch& bl);
+                           cudaStream_t s, BatchLaunch& bl, BatchRows& rows);
 // The launches of a batch whose particles per CTA are left to the library: the problems that run
 // best with one particle per CTA in one, those with two in another, which fills the SMs as the
 // first drains (the same bits either way).
@@ -161,9 +178,10 @@ struct BatchSet {
     BatchSet& operator=(const BatchSet&) = delete;
     ~BatchSet();
 };
-// cfg.particles_per_cta 0: as above; 1 or 2: one launch of that shape.
+// cfg.particles_per_cta 0: as above; 1 or 2: one launch of that shape.  rows: of the two launches, which run
+// side by side.
 spasm_status prepare_batches(spasm_problem_t* prs, const std::vector<int>& order, const spasm_batch_config& cfg,
-                             cudaStream_t s, BatchSet& set);
+                             cudaStream_t s, BatchSet& set, BatchRows rows[2]);
 spasm_status enqueue_batches(const BatchSet& set, cudaStream_t s);
 // Enqueues the launch (resetting its work counter first).
 spasm_status enqueue_batch(const BatchLaunch& bl, cudaStream_t s);

@@ -119,6 +119,7 @@ void scheduler_loop(spasm_server* sv) {
     cudaSetDevice(sv->device);
     cudaStream_t st = nullptr;
     if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) st = nullptr;
+    auto rows = std::make_unique<BatchRows[]>(2);   // the epochs' launches', whatever is in flight
     std::vector<std::shared_ptr<Request>> active;
     spasm_batch_config cfg;
     spasm_batch_default_config(&cfg);
@@ -143,7 +144,7 @@ void scheduler_loop(spasm_server* sv) {
         // new requests: problem, stage 1 (device-side attempt loop), first lift
         Range epoch_range("spasm service epoch");
         for (auto& r : admitted) {
-            int status = spasm_create_problem(&r->robot, &r->obs, &r->goal, &r->prm, st, &r->pr);
+            int status = create_served_problem(&r->robot, &r->obs, &r->goal, &r->prm, st, &r->pr);
             if (status == SPASM_OK) status = spasm_place(r->pr);
             if (status == SPASM_OK) status = enqueue_traj_lift(r->pr, st);
             if (status != SPASM_OK) {
@@ -166,7 +167,7 @@ void scheduler_loop(spasm_server* sv) {
         std::string msg;
         {
             BatchSet bl;
-            status = prepare_batches(prs.data(), order, cfg, st, bl);
+            status = prepare_batches(prs.data(), order, cfg, st, bl, rows.get());
             if (status == SPASM_OK) status = enqueue_batches(bl, st);
             for (auto& r : active)
                 if (status == SPASM_OK) status = enqueue_traj_epoch_end(r->pr, st);
@@ -223,6 +224,7 @@ void scheduler_loop(spasm_server* sv) {
         sv->cv_work.notify_all();
         sv->cv_done.notify_all();
     }
+    rows.reset();
     if (st) cudaStreamDestroy(st);
 }
 

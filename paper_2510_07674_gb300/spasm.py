@@ -351,7 +351,7 @@ def spasm_fp32_fma_peak(target_ms: float = 200.0) -> dict:
 
 
 def spasm_problem_bytes(workload, **overrides) -> int:
-    """Device bytes spasm_create_problem would allocate for this workload."""
+    """Device bytes of this workload's problem, without the scratch of its trajectory launches."""
     d = ProblemDesc(workload, **overrides)
     b = ctypes.c_longlong()
     _check(lib().spasm_problem_bytes(ctypes.byref(d._obs), ctypes.byref(d._goal), ctypes.byref(d._params), ctypes.byref(b)))
