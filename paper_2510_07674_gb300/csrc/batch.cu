@@ -293,17 +293,16 @@ spasm_status spasm::prepare_batches(spasm_problem_t* prs, const std::vector<int>
 }
 
 spasm_status spasm::enqueue_batches(const BatchSet& set, cudaStream_t s) {
-    if (set.side) {
-        SPASM_CUDA(cudaEventRecord(set.fork, s));
-        SPASM_CUDA(cudaStreamWaitEvent(set.side, set.fork, 0));
-    }
-    SPASM_TRY(enqueue_batch(set.launch[0], s));
-    if (set.side) {
-        SPASM_TRY(enqueue_batch(set.launch[1], set.side));
-        SPASM_CUDA(cudaEventRecord(set.join, set.side));
-        SPASM_CUDA(cudaStreamWaitEvent(s, set.join, 0));
-    }
-    return SPASM_OK;
+    if (!set.side) return enqueue_batch(set.launch[0], s);
+    SPASM_CUDA(cudaEventRecord(set.fork, s));
+    SPASM_CUDA(cudaStreamWaitEvent(set.side, set.fork, 0));
+    spasm_status st = enqueue_batch(set.launch[0], s);
+    if (st == SPASM_OK) st = enqueue_batch(set.launch[1], set.side);
+    // joined after a failure too: the work lists, and the problems, are given back on s
+    cudaError_t e = cudaEventRecord(set.join, set.side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, set.join, 0);
+    if (st == SPASM_OK) SPASM_CUDA(e);
+    return st;
 }
 
 extern "C" spasm_status spasm_batch_default_config(spasm_batch_config* cfg) {
