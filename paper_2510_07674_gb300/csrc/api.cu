@@ -386,6 +386,12 @@ static spasm_status create_problem_impl(const spasm_robot* robot, const spasm_ob
         for (int i = 0; i < B; ++i) turned = std::fmax(turned, std::fabs(q.init[i][3]) * norm3(q.half[i]));
         const double reach = arm + norm3(q.ee_p) + tip + held;
         q.margin = (float)(2e-5 * (reach + far) + 2.5e-7 * (offsets * reach + turned));
+        // A placed block's yaw is off by the rotation's error (at most a quarter of the margin, as a part of the
+        // extent) over the length l of its x axis in the plane, its corners by that times its half diagonal:
+        // no more than a quarter of the margin while l is at least half diagonal / extent
+        double diagonal = 0.0;
+        for (int i = 0; i < B; ++i) diagonal = std::fmax(diagonal, std::hypot(q.half[i][0], q.half[i][1]));
+        q.level2 = (float)std::pow(diagonal / (reach + far), 2.0);
     }
     pr->host_osph.assign(obs->sphere, obs->sphere + 4 * (size_t)sc.n_osph);
 

@@ -83,8 +83,6 @@ constexpr int kScrCfgs = 4 * kScrWarps;   // configurations per CTA of the scree
 constexpr int kChkThreads = 128, kChkWarps = kChkThreads / 32;
 constexpr float kNone = -3.4e38f;         // no obstacle within the margin
 constexpr float kMaxAngle = 8.f;          // largest joint value the FP32 evaluation takes
-constexpr float kMinLevel2 = 0.25f;       // least squared horizontal part of a placed block's x axis (unit length):
-                                          // the yaw's error is at most twice the rotation's
 
 struct ScreenWarp {
     float4 F[4][8][3];   // frames 0..7 of the warp's configurations: rows (R_i0, R_i1, R_i2, o_i)
@@ -285,7 +283,7 @@ __global__ void __launch_bounds__(kScrThreads) k_check_screen(const __grid_const
             if (k == 7) {
                 tool_frame<float>(sc, R, o, Rt, pt);
                 held_block<float>(sc, b, Rt, pt, Rb, pb);
-                if (joints || !(Rb[0] * Rb[0] + Rb[3] * Rb[3] >= kMinLevel2)) atomicOr(&sh.loose, 1u << b);
+                if (joints || !(Rb[0] * Rb[0] + Rb[3] * Rb[3] >= s.level2)) atomicOr(&sh.loose, 1u << b);
                 block_cuboid(pb[0], pb[1], pb[2], atan2f(Rb[3], Rb[0]), sc.half[b], sh.blk[b]);
                 cuboid_box(sh.blk[b], sh.box[n_env + b]);
             }

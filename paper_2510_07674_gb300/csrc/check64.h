@@ -17,6 +17,7 @@ struct Scalars64 {
     double grasp_off, eps, eps_start;
     int p2p;   // point to point: one segment, no placement
     float margin;   // bound on the error of a sphere-obstacle distance evaluated in FP32
+    float level2;   // least squared horizontal part of a placed block's x axis (unit length) for it to hold
 };
 
 // Per-solution accumulator of the check (zeroed once at allocation; the check leaves its

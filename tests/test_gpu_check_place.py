@@ -14,6 +14,9 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 B, W, N_TRAJ = 3, 8, 24
+# horizontal part of the x axis: FP32 gives no yaw at all; and on both sides of the least that it is trusted
+# with (half diagonal / extent of the scene, here about 0.01)
+LEVEL = {"vertical": lambda rng: 2e-6, "tilted": lambda rng: 10.0 ** rng.uniform(-3.0, -1.0)}
 
 
 def _workload(offsets=0.0):
@@ -24,10 +27,10 @@ def _workload(offsets=0.0):
     return wl
 
 
-def _upright(orc, rng):
-    """A configuration whose tool x axis is vertical up to 2e-6: Newton steps on its horizontal part."""
+def _upright(orc, rng, level):
+    """A configuration whose tool x axis is vertical up to `level`: Newton steps on its horizontal part."""
     angle = rng.uniform(-np.pi, np.pi)
-    target = 2e-6 * np.array([np.cos(angle), np.sin(angle)])
+    target = level * np.array([np.cos(angle), np.sin(angle)])
 
     def res(q):
         return orc.fk(q)[1][:2, 0] - target
@@ -53,13 +56,13 @@ def _trajectories(kind, wl, orc):
             q[p, t] = far.astype(np.float32)
             near = np.mod(q[p, t] + np.pi, 2 * np.pi) - np.pi   # the same angles
         else:
-            q[p, t] = near = _upright(orc, rng)
+            q[p, t] = near = _upright(orc, rng, LEVEL[kind](rng))
         spread = 0.08 if kind == "large" else 0.01
         q[p, t + 1:] = near + rng.uniform(-spread, spread, (C - t - 1, 7))
     return q
 
 
-@pytest.mark.parametrize("kind", ["large", "vertical"])
+@pytest.mark.parametrize("kind", ["large", "vertical", "tilted"])
 def test_placed_blocks_that_fp32_cannot_place(kind):
     from paper_2510_07674_gb300 import spasm as S
     wl = _workload(np.array([0.3, -0.7, 1.1, -0.2, 0.9, -1.3, 0.5]) if kind == "large" else 0.0)
