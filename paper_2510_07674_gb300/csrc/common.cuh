@@ -157,12 +157,6 @@ __device__ __forceinline__ float warp_max(float v) {
     return v;
 }
 
-__device__ __forceinline__ float warp_min(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
 // Smallest / largest of the lanes' values (NaN ignored, as fminf / fmaxf) in one instruction.
 __device__ __forceinline__ float warp_fmin(float v) {
     float r;
@@ -307,9 +301,6 @@ __device__ __forceinline__ void dh_step(T R[9], T o[3], T ca, T sa, T a, T d, T 
     for (int i = 0; i < 9; ++i) R[i] = n[i];
 }
 
-__device__ __forceinline__ void sincos_t(float x, float* s, float* c) { sincosf(x, s, c); }
-__device__ __forceinline__ void sincos_t(double x, double* s, double* c) { sincos(x, s, c); }
-
 // Tool frame from frame 7: R_tool = R7 ee_R, p_tool = o7 + R7 ee_p.
 template <typename T>
 __device__ __forceinline__ void tool_frame(const TrajScalars& sc, const T R7[9], const T o7[3], T Rt[9], T pt[3]) {
@@ -320,24 +311,6 @@ __device__ __forceinline__ void tool_frame(const TrajScalars& sc, const T R7[9],
             Rt[3 * i + j] = R7[3 * i] * (T)sc.ee_R[j] + R7[3 * i + 1] * (T)sc.ee_R[3 + j] + R7[3 * i + 2] * (T)sc.ee_R[6 + j];
         pt[i] = o7[i] + R7[3 * i] * (T)sc.ee_p[0] + R7[3 * i + 1] * (T)sc.ee_p[1] + R7[3 * i + 2] * (T)sc.ee_p[2];
     }
-}
-
-// Full FK of one configuration: frames 1..7 as (R, o), and the tool frame.
-template <typename T>
-__device__ __forceinline__ void fk_full(const Scalars& sc, const T q[7], T R[8][9], T o[8][3], T Rt[9], T pt[3]) {
-#pragma unroll
-    for (int i = 0; i < 9; ++i) R[0][i] = (i % 4 == 0) ? (T)1 : (T)0;
-    o[0][0] = o[0][1] = o[0][2] = (T)0;
-#pragma unroll
-    for (int k = 0; k < 7; ++k) {
-        T s, c;
-        sincos_t((T)sc.th0[k] + q[k], &s, &c);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) R[k + 1][i] = R[k][i];
-        o[k + 1][0] = o[k][0]; o[k + 1][1] = o[k][1]; o[k + 1][2] = o[k][2];
-        dh_step<T>(R[k + 1], o[k + 1], (T)sc.ca[k], (T)sc.sa[k], (T)sc.a[k], (T)sc.d[k], c, s);
-    }
-    tool_frame<T>(sc, R[7], o[7], Rt, pt);
 }
 
 // Block frame held by the tool (top-down grasp): R_blk = R_tool diag(1,-1,-1),

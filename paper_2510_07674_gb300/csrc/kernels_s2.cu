@@ -794,7 +794,7 @@ __device__ __forceinline__ void placed_slice(const TrajScalars& sc, const float4
 }
 
 // Modes of the trajectory kernel
-enum TrajMode { kTrajEval = 0, kTrajDescend = 1, kTrajCheck = 2 };
+enum TrajMode { kTrajEval = 0, kTrajDescend = 1 };
 
 // Axis-aligned box of a cuboid record (centre, then R columns with half extents).
 __device__ __forceinline__ void cuboid_aabb(const float4* c, float4* box) {

@@ -40,7 +40,7 @@ struct TrajIO {
 constexpr int kTrajSlots = 608;
 constexpr size_t kHalfSmem = 228 * 512 - 1024;   // shared memory of each of two CTAs on an SM
 int traj_slots(int B, int C, int n_cub, int n_osph);
-enum TrajModeHost { kTrajModeEval = 0, kTrajModeDescend = 1, kTrajModeCheck = 2 };
+enum TrajModeHost { kTrajModeEval = 0, kTrajModeDescend = 1 };
 
 // One problem of a batched trajectory launch (device array, sorted by `first`).
 struct TrajJob {
