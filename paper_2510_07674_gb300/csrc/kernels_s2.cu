@@ -983,7 +983,7 @@ __device__ void traj_evaluate(const TrajScalars& sc, const LaneSpheres& ls, cons
                 // point, which has none, takes the start residuals here
                 float my_D = 0.f, my_e = 0.f;
                 if (p2p) start_job();
-                else place_stack_warp(sc, sh.pose, kPlaceUnit, nullptr, nullptr, nullptr, sh.ps, sh.blk, my_D, my_e);
+                else place_stack_warp(sc, sh.pose, kPlaceUnit, nullptr, sh.ps, sh.blk, my_D, my_e);
                 const float c_stable = warp_sum(lane < B ? my_D : 0.f);
                 const float c_height = warp_sum(lane < B ? my_e * my_e : 0.f);
                 const float max_D = warp_fmax(lane < B ? my_D : 0.f);

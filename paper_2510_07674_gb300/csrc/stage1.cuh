@@ -30,21 +30,19 @@ struct PlaceScratch : StackScratch {
     float4 bc[kMaxB][4];     // block cuboids
 };
 
-// Coefficient modes of the gradient: stage-1 cost (a = w_stable, b = 2 w_height e,
-// s_coll = w_coll), explicit per-residual coefficients (stage 2), or the residuals with the
-// unit-coefficient support factors (a = 1) left in ps.stab and no gradient written (stage 2
-// scales them by its multipliers once those are known).
-enum PlaceMode { kPlaceForward = 0, kPlaceStage1 = 1, kPlaceExplicit = 2, kPlaceUnit = 3 };
+// Coefficient modes of the gradient: none, stage-1 cost (a = w_stable, b = 2 w_height e), or the
+// residuals with the unit-coefficient support factors (a = 1) left in ps.stab and no gradient
+// written (stage 2 scales them by its multipliers once those are known).
+enum PlaceMode { kPlaceForward = 0, kPlaceStage1 = 1, kPlaceUnit = 2 };
 
 // Per-block terms of the tower (lane i < B owns block i): height residual e_i, support
-// distance D_i and the block cuboids in ps.  With mode kPlaceStage1 or kPlaceExplicit, sets
+// distance D_i and the block cuboids in ps.  With mode kPlaceStage1, sets
 //   g = sum_i a_i dD_i/dx + sum_i b_i de_i/dx   (the collision part is added by the caller);
 // with kPlaceUnit, leaves dD_i/d(centre of mass, yaw) in ps.stab for place_stack_grad.
 // x, g: per-warp shared arrays of 4B floats.  Must be called by all 32 lanes of the warp.
 // bc: the block cuboids, written here or, in mode kPlaceUnit, already those of x.
-__device__ __forceinline__ void place_stack_warp(const TrajScalars& sc, const float* x, int mode, const float* a_in,
-                                                 const float* b_in, float* g, StackScratch& ps, float4 (*bc)[4],
-                                                 float& my_D, float& my_e) {
+__device__ __forceinline__ void place_stack_warp(const TrajScalars& sc, const float* x, int mode, float* g,
+                                                 StackScratch& ps, float4 (*bc)[4], float& my_D, float& my_e) {
     const int lane = threadIdx.x & 31;
     const int B = sc.B;
     const bool want_grad = mode != kPlaceForward;
@@ -66,7 +64,7 @@ __device__ __forceinline__ void place_stack_warp(const TrajScalars& sc, const fl
             const float ex = fmaxf(fabsf(ux) - sc.half[i].x, 0.f), ey = fmaxf(fabsf(uy) - sc.half[i].y, 0.f);
             my_D = sqrtf(ex * ex + ey * ey);
             if (want_grad && my_D > 0.f) {
-                const float a = mode == kPlaceStage1 ? sc.w_stable : mode == kPlaceUnit ? 1.f : a_in[i];
+                const float a = mode == kPlaceStage1 ? sc.w_stable : 1.f;
                 const float du_x = (ux >= 0.f ? ex : -ex) / my_D, du_y = (uy >= 0.f ? ey : -ey) / my_D;
                 dvx = a * (c * du_x - s * du_y);
                 dvy = a * (s * du_x + c * du_y);
@@ -85,14 +83,14 @@ __device__ __forceinline__ void place_stack_warp(const TrajScalars& sc, const fl
             gx += ps.stab[k][0] * inv;
             gy += ps.stab[k][1] * inv;
         }
-        const float b = mode == kPlaceStage1 ? 2.f * sc.w_height * my_e : b_in[i];
+        const float b = 2.f * sc.w_height * my_e;
         g[4 * i] = gx; g[4 * i + 1] = gy; g[4 * i + 2] = b; g[4 * i + 3] = ps.stab[i][2];
     }
     __syncwarp();
 }
 
-// The gradient place_stack_warp writes in mode kPlaceExplicit, from the factors its kPlaceUnit
-// pass left in ps (a_i dD_i/d... = a_i times the unit factor, in the same order of operations).
+// sum_i a_i dD_i/dx + sum_i b_i de_i/dx for coefficients a_in, b_in, from the unit factors that
+// place_stack_warp's kPlaceUnit pass left in ps.
 // inv_above[k] = 1 / (B - 1 - k), the blocks above block k < B - 1.
 __device__ __forceinline__ void place_stack_grad(const TrajScalars& sc, const StackScratch& ps, const float* a_in,
                                                  const float* b_in, const float* inv_above, float* g) {
@@ -159,17 +157,16 @@ __device__ __forceinline__ float group_sums(float v0, float v1, float v2, float 
 // cand: per-warp scratch of kMaxCub/32 + kMaxOSph/32 words (the candidate obstacles of the particle).
 __device__ __forceinline__ void place_eval_warp(const Scalars& sc, const float4* __restrict__ cub, int n_cub,
                                                 const float4* __restrict__ osph, int n_osph, const float* x,
-                                                bool quad, int mode, const float* a_in, const float* b_in,
-                                                float s_coll_in, float* g, PlaceScratch& ps, uint32_t* cand,
+                                                bool quad, int mode, float* g, PlaceScratch& ps, uint32_t* cand,
                                                 PlaceOut* out) {
     const int lane = threadIdx.x & 31;
     const int B = sc.B;
     const bool want_grad = mode != kPlaceForward;
     float my_D, my_e;
-    place_stack_warp(sc, x, mode, a_in, b_in, g, ps, ps.bc, my_D, my_e);
+    place_stack_warp(sc, x, mode, g, ps, ps.bc, my_D, my_e);
 
     // -- collisions: items (block j, sphere m)
-    const float s_coll = mode == kPlaceStage1 ? sc.w_coll : s_coll_in;
+    const float s_coll = sc.w_coll;
     float coll = 0.f, maxpen = 0.f;
     const int n_items = 8 * B;
     // exact cull: the box of every block sphere of the particle (padded by 1e-5 against the

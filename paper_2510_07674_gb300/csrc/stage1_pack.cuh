@@ -27,9 +27,8 @@ namespace spasm {
 __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const float4* __restrict__ cub,
                                                      const float4* __restrict__ wall, int n_cub,
                                                      const float4* __restrict__ osph, int n_osph, const float* x,
-                                                     bool quad, int mode, const float* b_in, float s_coll_in,
-                                                     float* g, PlaceScratch& ps, float4* gcell, float4* cube,
-                                                     PlaceOut* out) {
+                                                     bool quad, int mode, float* g, PlaceScratch& ps, float4* gcell,
+                                                     float4* cube, PlaceOut* out) {
     const int lane = threadIdx.x & 31;
     const int B = sc.B;
     const bool want_grad = mode != kPlaceForward;
@@ -43,7 +42,7 @@ __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const fl
         my_e = x[4 * i + 2] - sc.z_star;
         block_cuboid(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3], half, ps.bc[i]);
         if (want_grad) {
-            const float b = mode == kPlaceStage1 ? sc.w_height * (my_e > 0.f ? 1.f : (my_e < 0.f ? -1.f : 0.f)) : b_in[i];
+            const float b = sc.w_height * (my_e > 0.f ? 1.f : (my_e < 0.f ? -1.f : 0.f));
             g[4 * i] = 0.f; g[4 * i + 1] = 0.f; g[4 * i + 2] = b; g[4 * i + 3] = 0.f;
         }
     }
@@ -57,7 +56,7 @@ __device__ __forceinline__ void place_eval_pack_warp(const Scalars& sc, const fl
     }
     __syncwarp();
 
-    const float s_coll = mode == kPlaceStage1 ? sc.w_coll : s_coll_in;
+    const float s_coll = sc.w_coll;
     float coll = 0.f, maxpen = 0.f;
     const int n_items = 8 * sc.n_cells;
     for (int base = 0; base < n_items; base += 32) {
@@ -189,9 +188,9 @@ __device__ __forceinline__ void place_eval(const Scalars& sc, const float4* __re
                                            int mode, float* g, PlaceScratch& ps, float4* gcell, float4* cube,
                                            uint32_t* cand, PlaceOut* out) {
     if (!kTower && sc.kind == kKindPack)
-        place_eval_pack_warp(sc, cub, wall, n_cub, osph, n_osph, x, quad, mode, nullptr, 0.f, g, ps, gcell, cube, out);
+        place_eval_pack_warp(sc, cub, wall, n_cub, osph, n_osph, x, quad, mode, g, ps, gcell, cube, out);
     else
-        place_eval_warp(sc, cub, n_cub, osph, n_osph, x, quad, mode, nullptr, nullptr, 0.f, g, ps, cand, out);
+        place_eval_warp(sc, cub, n_cub, osph, n_osph, x, quad, mode, g, ps, cand, out);
 }
 
 }  // namespace spasm
