@@ -364,7 +364,7 @@ def run_native(args, ws, rank, local):
     nominal = SM_COUNT * FP32_LANES * 2 * clk * 1e6 / 1e12
     peak = fp32_peak["tflops"]
     traffic = traffic_from_profile()
-    roofline = {"bound": "alu", "kernel": "k_traj (fused stage-2 descent, one CTA per particle)",
+    roofline = {"bound": "alu", "kernel": "k_traj (fused stage-2 descent, a group of 8, 4 or 2 warps per particle)",
                 "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": (achieved / peak) if achieved else None,
                 "traffic": traffic,
                 "peak_basis": (f"measured: FP32 FMA chains on every SM (spasm_fp32_fma_peak), "

@@ -436,8 +436,9 @@ spasm_status spasm_optimize_batch(spasm_problem_t* problems, int n, void* cuda_s
  * CTA in {1, 2}, where its shared memory fits) over one full descent of every particle, then,
  * under the fastest shape, one evaluation of every particle per schedule (per_fetch in
  * {1, 2, 4} x ctas_per_sm in {all, 1} x both orders; CUDA events, the better of two runs), and
- * returns the fastest in *best (and that schedule's evaluation time in *best_ms when not
- * NULL).  The tuning writes only buffers a solve sets again (the particles are lifted again
+ * returns the fastest of these in *best (and that schedule's evaluation time in *best_ms when
+ * not NULL).  Each is one shape for the whole batch: a batch on both sides of the library's own
+ * rule (up to 6 blocks and more) can be faster with cfg NULL.  The tuning writes only buffers a solve sets again (the particles are lifted again
  * and the multipliers start fresh).  The schedule and the particles per CTA change no result;
  * the sphere tiling changes results at float32 rounding. */
 spasm_status spasm_batch_autotune(spasm_problem_t* problems, int n, void* cuda_stream, spasm_batch_config* best,

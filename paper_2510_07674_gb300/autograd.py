@@ -8,7 +8,10 @@ backward, which shares the kinematics, the culls and the residuals with the cost
 gradient (the size of the input; no transforms are stored); the backward pass scales it by the
 incoming gradient, particle by particle.  A second kernel run in the backward pass, with
 everything computed again, took 2.36 ms in place of 1.29 ms for 4096 trajectories of the
-10-block tower.  Without a gradient to compute the forward pass runs the kernel without its backward part.
+10-block tower.  Without a gradient to compute the forward pass runs the kernel without its backward part;
+a caller who wants only the value of an input that requires a gradient says so with torch.no_grad()
+(without it the call holds a tensor of the input's size and takes 1.15 in place of 1.06 ms there, 38 in
+place of 28 us for a few placements).
 Inputs are CUDA float32 tensors; no computation happens in Python.
 """
 from __future__ import annotations

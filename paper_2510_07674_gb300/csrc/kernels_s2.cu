@@ -1,5 +1,5 @@
-// Stage-2 kernels: the fused trajectory optimisation (one CTA per particle, every
-// iteration inside one launch).  The lift that initialises it is in kernels_lift.cu.
+// Stage-2 kernels: the fused trajectory optimisation (a group of 8, 4 or 2 warps per particle,
+// every iteration inside one launch).  The lift that initialises it is in kernels_lift.cu.
 #include <algorithm>
 
 #include <cuda_fp16.h>
@@ -1244,8 +1244,8 @@ template <int kPpc>
 __device__ __forceinline__ void traj_path(const TrajScalars& sc, TShared& sh, const float* q) {
     const int tid = grp_tid<kPpc>(), lane = tid & 31, w = tid >> 5;
     const int C = sc.C;
-    // partial sums in the order of 256 threads, whatever the group: thread tid holds those of
-    // threads tid and, with two groups, tid + 128
+    // partial sums in the order of 256 threads, whatever the group: thread tid of kGrpThreads holds
+    // those of threads tid, tid + kGrpThreads, ...
     float path[kPpc], jl[kPpc];
 #pragma unroll
     for (int i = 0; i < kPpc; ++i) {
@@ -1616,12 +1616,13 @@ static cudaError_t sm_limits(int* sms, size_t* half_smem) {
 // hold one CTA, 8 warps in place of 16).
 // Towers of more than kAutoBlocks blocks keep one: their phases run through more of the kernel's
 // code at a time, and four particles in different phases miss the instruction cache.  4096
-// particles, 50 steps, one / two per CTA, ms: 2 blocks 4.1 / 2.7, 4 blocks 5.6 / 4.0, 6 blocks
-// 6.9 / 5.8, 8 blocks 9.2 / 9.0, 10 blocks 12.6 / 15.5.
+// particles among 64 cuboids, 50 steps, one / two per CTA, ms: 2 blocks 4.1 / 2.8, 4 blocks
+// 5.6 / 4.1, 6 blocks 7.6 / 6.7, 8 blocks 9.5 / 9.9, 10 blocks 13.8 / 17.7.
 // Four take short trajectories (kShortC configurations; 1 block, 31 configurations, 700 / 4096
-// particles, two / four per CTA: 0.82 / 0.68 and 2.62 / 1.86 ms), and longer ones up to kMidC when
+// particles, two / four per CTA: 0.56 / 0.35 and 1.94 / 1.30 ms), and longer ones up to kMidC when
 // the launch has several rounds of them, as a particle on two warps runs long and the last ones
-// run alone (3 blocks, 187 configurations, 2048 / 4096 particles: 2.86 / 3.33 and 4.75 / 4.35 ms).
+// run alone (3 blocks, 187 configurations, 4096 particles: 3.44 / 2.70 ms; at 2048, where the line
+// keeps two, 1.91 / 1.55, but 2.86 / 3.33 where more of the chunks have candidates).
 // cta_bytes_2, cta_bytes_4: the shared memory of a CTA with 2 or 4 particles (0: not to be used).
 constexpr int kAutoBlocks = 6, kShortC = 48, kMidC = 192;
 int traj_auto_ppc(size_t cta_bytes_2, size_t cta_bytes_4, long long particles, int blocks, int C) {
@@ -1667,8 +1668,10 @@ int traj_batch_ctas_per_sm(size_t cta_bytes, int tiling, int ppc) {
 
 int traj_ppc(const TrajScalars& sc, long long particles) {
     if (sc.particles_per_cta) return sc.particles_per_cta;
-    // point to point keeps two (1024 / 4096 particles, two / four per CTA: 1.9 / 2.3 and 5.9 / 5.8 ms):
-    // its eight chunks, all near obstacles, are too few and too long for two warps
+    // point to point keeps two: its chunks, all near obstacles, are long for two warps, unless they are
+    // few (50 steps, 1024 / 4096 particles, two / four per CTA, ms: 32 configurations 1.57 / 1.80 and
+    // 4.46 / 4.28, 64 configurations 2.73 / 2.91 and 8.27 / 7.93, 8 configurations 0.53 / 0.39 and
+    // 1.59 / 1.03)
     const bool four = !sc.sphere_tiling && sc.kind != kKindP2P;
     return traj_auto_ppc(traj_cta_smem_bytes(sc, 2, false), four ? traj_cta_smem_bytes(sc, 4, false) : 0, particles, sc.B,
                          sc.C);
