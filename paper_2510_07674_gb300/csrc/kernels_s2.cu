@@ -1679,7 +1679,8 @@ int traj_ppc(const TrajScalars& sc, long long particles) {
 
 template <bool kP2P>
 static int single_ctas(size_t dyn, int tiling, int ppc) {
-    if (ppc == 4) return occupancy(k_traj<kP2P, 0, 4>, dyn);
+    if constexpr (!kP2P)   // point to point never takes four (traj_ppc)
+        if (ppc == 4) return occupancy(k_traj<false, 0, 4>, dyn);
     if (ppc == 2) return tiling ? occupancy(k_traj<kP2P, 1, 2>, dyn) : occupancy(k_traj<kP2P, 0, 2>, dyn);
     return tiling ? occupancy(k_traj<kP2P, 1, 1>, dyn) : occupancy(k_traj<kP2P, 0, 1>, dyn);
 }
@@ -1715,7 +1716,8 @@ static cudaError_t traj_dispatch(const Scalars& sc, DevTables t, int n, int mode
         const size_t env = t_env_bytes(sc.n_cub, sc.n_osph), rows = t_rows_bytes(sc.C);
         while (ppc > 1 && env + ppc * (t_region(sc.C, sc.B, ppc) + rows) > kHalfSmem) ppc /= 2;
     }
-    if (ppc == 4) return traj_kernel<kP2P, 0, 4>(sc, t, n, mode, io, err, st);
+    if constexpr (!kP2P)
+        if (ppc == 4) return traj_kernel<false, 0, 4>(sc, t, n, mode, io, err, st);
     if (ppc == 2)
         return sc.sphere_tiling ? traj_kernel<kP2P, 1, 2>(sc, t, n, mode, io, err, st)
                                 : traj_kernel<kP2P, 0, 2>(sc, t, n, mode, io, err, st);

@@ -5,21 +5,36 @@ groups that are resident.)"""
 import numpy as np
 import pytest
 
+from paper_2510_07674_gb300 import scenes
 from test_gpu_traj_groups import _lifted, _problem, _run, _same
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("size, n", [((1, 4, 0, 12), 1300), ((3, 12, 5, 9), 700), ((3, 255, 64, 32), 2500),
+def _point_to_point(n):
+    from paper_2510_07674_gb300 import spasm as S
+    pr = S.Problem(scenes.make_p2p("p2p", seed=5, O=30, W=20, Q=16))
+    rng = np.random.default_rng(4)
+    ends = np.asarray(scenes.make_robot(7).q_home) + rng.uniform(-0.9, 0.9, (n, 2, 7))
+    path = ends[:, :1] + np.linspace(0, 1, pr.C)[None, :, None] * (ends[:, 1:] - ends[:, :1])
+    q = torch.zeros(n, pr.C, 8, device="cuda")
+    q[:, :, :7] = torch.from_numpy(path.astype(np.float32)).cuda()
+    return S, pr, q
+
+
+@pytest.mark.parametrize("size, n", [(None, 700), ((1, 4, 0, 12), 1300), ((3, 12, 5, 9), 700), ((3, 255, 64, 32), 2500),
                                      ((6, 20, 0, 32), 700), ((16, 255, 64, 32), 330)])
 def test_captured_calls_replayed_side_by_side(size, n):
     cap, a, b = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.Stream()
     with torch.cuda.stream(cap):
-        S, pr = _problem(*size)
+        if size is None:
+            S, pr, q = _point_to_point(2 * n)
+        else:
+            S, pr = _problem(*size)
+            q = _lifted(S, pr, 2 * n)
         try:
             gen = torch.Generator().manual_seed(2)
-            q = _lifted(S, pr, 2 * n)
             lam, mu = torch.rand(2 * n, pr.NR, generator=gen).cuda(), 1 + torch.rand(2 * n, generator=gen).cuda()
             torch.cuda.synchronize()
             ref = _run(S, pr, q, lam, mu)
